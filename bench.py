@@ -221,13 +221,14 @@ class ClockSampler:
 
 # the sources the 2D step's kernels, their launch shapes and tile lists are
 # built from (the 3D, network and allocation-free units do not enter)
-_SWEEP_SOURCES = ["fvna_api.cu", "fvna_device.cuh", "fvna_fp32.cu", "fvna_fp64.cu",
+_SWEEP_SOURCES = ["fvna_api.cu", "fvna_device.cuh", "fvna_face64.cuh", "fvna_fp32.cu",
+                  "fvna_fp64.cu", "fvna_int64f.cuh", "fvna_sweeps64.cuh",
                   "fvna_launch.h", "fvna_precision.inc", "fvna_step.cuh", "fvna_sweeps.cuh",
                   "fvna_sweeps32.cuh", "fvna_types.h", "fvna_x2.cuh"]
 
 
 _SWEEP3_SOURCES = ["fvna_3d.cuh", "fvna_3d.inc", "fvna_3d32.cu", "fvna_3d64.cu", "fvna_api3d.cu",
-                   "fvna_launch3.h"]
+                   "fvna_face64.cuh", "fvna_int64f.cuh", "fvna_launch3.h"]
 
 
 def source_digest(files=None):
@@ -258,8 +259,8 @@ def ncu_traffic(kernel_key: str, files=None):
 _TRAFFIC_KEYS = [
     (r"k_sweep_x32<", "k_sweep_x_fp32"),
     (r"k_sweep_y32<", "k_sweep_y_fp32"),
-    (r"k_sweep_x<(fvna::)?P64", "k_sweep_x_fp64"),
-    (r"k_sweep_y<(fvna::)?P64", "k_sweep_y_fp64"),
+    (r"k_sweep_x64<", "k_sweep_x_fp64"),
+    (r"k_sweep_y64<", "k_sweep_y_fp64"),
 ]
 # the 3D kernels (k3_sweep_v serves the x2 and the x3 sweep: one figure for both)
 _TRAFFIC_KEYS3 = [

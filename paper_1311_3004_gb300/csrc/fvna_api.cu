@@ -43,8 +43,8 @@ struct fvna_ctx {
   int tile_x = 32, tile_y = 64;
   int blocks_x = 1, blocks_y = 1;
   StepArgs args;    // common arguments (no tile list)
-  StepArgs args_x;  // x1 sweep: warp tiles of 32 rows x tile_x cells
-  StepArgs args_y;  // x2 sweep: warp tiles of 30 columns x tile_y rows
+  StepArgs args_x;  // with the x1 sweep's warp tiles
+  StepArgs args_y;  // with the x2 sweep's
   DomScal *h_scal = nullptr;  // pinned mirror
   long long launches = 0;
   int kernels_per_step = 3;
@@ -372,9 +372,13 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
   int dev = 0, sms = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  Tiles64 t64 = {};
   if (prec == FVNA_FP64) {
-    c->tile_x = cfg->tile_x ? cfg->tile_x : 32;
-    c->tile_y = cfg->tile_y ? cfg->tile_y : 64;
+    std::vector<Extent> ext(n);
+    for (int d = 0; d < n; d++) ext[d] = Extent{doms[d].nx, doms[d].ny};
+    pick_tiles64(n, ext.data(), sms, cfg->limiter, cfg->tile_x, cfg->tile_y, &t64);
+    c->tile_x = t64.tile_x;
+    c->tile_y = t64.tile_y;
   } else {
     c->tile_x = cfg->tile_x ? cfg->tile_x : pick_tile_x32(n, doms, sms);
     c->tile_y = cfg->tile_y ? cfg->tile_y : pick_tile_y32();
@@ -452,7 +456,8 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
   CK(cudaMemcpyAsync(c->d_scal, sc.data(), sizeof(DomScal) * n, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMallocHost(&c->h_scal, sizeof(DomScal) * n));
 
-  // warp tiles (binary64: 32 rows x tile_x and 30 columns x tile_y;
+  // warp tiles (binary64: segments of one or two cells a lane, some rows of
+  // them, and 30 columns x tile_y;
   // binary32: 32 rows x 2 halves and 60 columns x tile_y)
   // (binary32: the tiles that touch a domain border come first; they take
   // longer and the sweeps hand tiles out in list order)
@@ -460,41 +465,50 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
   const int sw = x32_half(c->tile_x);
   // binary32 x1 sweep with the lanes along x1: segments of two rows x 60 cells
   const bool xh = prec == FVNA_FP32_PERT && c->tile_x == X32H_TILE;
-  const int xstep = prec == FVNA_FP64 ? c->tile_x : xh ? X32H_TILE : 2 * sw;
-  const int xrows = xh ? 2 : XROWS;
-  const int ystep = prec == FVNA_FP64 ? YCOLS : Y32_COLS;
-  for (int d = 0; d < n; d++) {
+  const int xstep = prec == FVNA_FP64 ? x64_cells(c->tile_x) : xh ? X32H_TILE : 2 * sw;
+  const int xrows = prec == FVNA_FP64 ? t64.rows_x : xh ? 2 : XROWS;
+  const int ystep = prec == FVNA_FP64 ? t64.w_y : Y32_COLS;
+  // one binary64 domain: the kernels work the tiles out, no list
+  const bool listed = prec != FVNA_FP64 || n > 1;
+  for (int d = 0; d < n && listed; d++) {
     const int nx = doms[d].nx, ny = doms[d].ny;
     for (int y = 0; y < ny; y += xrows)
       for (int x = 0; x < nx; x += xstep) {
         bool b = xh ? (x < 2 || x + X32H_TILE + 2 > nx || y + 2 > ny)
                     : prec == FVNA_FP32_PERT && (x == 0 || x + 2 * sw + 2 > nx || y + XROWS > ny);
-        (b ? txb : tx).push_back(Tile{d, x, y, 0});
+        (b ? txb : tx).push_back(Tile{d, x, y, xrows});
       }
     for (int y = 0; y < ny; y += c->tile_y)
       for (int x = 0; x < nx; x += ystep) {
         bool b = prec == FVNA_FP32_PERT &&
                  (x < 2 || x + Y32_COLS + 2 > nx || y < HALO_Y || y + c->tile_y + HALO_Y > ny);
-        (b ? tyb : ty).push_back(Tile{d, x, y, 0});
+        (b ? tyb : ty).push_back(Tile{d, x, y, prec == FVNA_FP64 ? c->tile_y : 0});
       }
   }
   tx.insert(tx.begin(), txb.begin(), txb.end());
   ty.insert(ty.begin(), tyb.begin(), tyb.end());
-  c->ntx = (int)tx.size();
-  c->nty = (int)ty.size();
-  CK(cudaMalloc(&c->d_tx, sizeof(Tile) * tx.size()));
-  CK(cudaMalloc(&c->d_ty, sizeof(Tile) * ty.size()));
-  CK(cudaMemcpyAsync(c->d_tx, tx.data(), sizeof(Tile) * tx.size(), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemcpyAsync(c->d_ty, ty.data(), sizeof(Tile) * ty.size(), cudaMemcpyHostToDevice, c->stream));
+  if (listed) {
+    c->ntx = (int)tx.size();
+    c->nty = (int)ty.size();
+    CK(cudaMalloc(&c->d_tx, sizeof(Tile) * tx.size()));
+    CK(cudaMalloc(&c->d_ty, sizeof(Tile) * ty.size()));
+    CK(cudaMemcpyAsync(c->d_tx, tx.data(), sizeof(Tile) * tx.size(), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(c->d_ty, ty.data(), sizeof(Tile) * ty.size(), cudaMemcpyHostToDevice, c->stream));
+  } else {
+    c->ntx = ((doms[0].nx + xstep - 1) / xstep) * ((doms[0].ny + xrows - 1) / xrows);
+    c->nty = ((doms[0].nx + ystep - 1) / ystep) * ((doms[0].ny + c->tile_y - 1) / c->tile_y);
+  }
 
   // kernel set-up and persistent grid sizes
   const int comp = prec == FVNA_FP32_PERT && cfg->compensated ? 1 : 0;
   CK(prepare_kernels(prec, c->tile_x, cfg->limiter, comp));
   int occx = std::max(1, occupancy_x(prec, c->tile_x, cfg->limiter, comp));
-  int occy = std::max(1, occupancy_y(prec, cfg->limiter, comp));
-  const int wpb = prec == FVNA_FP64 ? WARPS_PER_BLOCK : 1;  // binary32: one warp per block
-  c->blocks_x = std::max(1, std::min((c->ntx + wpb - 1) / wpb, occx * sms));
-  c->blocks_y = std::max(1, std::min((c->nty + wpb - 1) / wpb, occy * sms));
+  if (prec == FVNA_FP64) {
+    c->blocks_x = std::min((c->ntx + WARPS_PER_BLOCK - 1) / WARPS_PER_BLOCK, occx * sms);
+  } else {   // one warp per block
+    c->blocks_x = std::max(1, std::min(c->ntx, occx * sms));
+    c->blocks_y = std::max(1, std::min(c->nty, std::max(1, occupancy_y(prec, cfg->limiter, comp)) * sms));
+  }
   if (prec == FVNA_FP32_PERT) {
     CK(build_maps_fp32(c->dd.data(), n, c->tile_x, &c->d_maps, c->stream));
     CK(cudaMalloc(&c->d_ctr, 3 * sizeof(unsigned)));
@@ -522,12 +536,18 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
   c->args_x = a;
   c->args_x.tiles = c->d_tx;
   c->args_x.ntiles = c->ntx;
+  c->args_x.tile_w = xstep;
+  c->args_x.tile_h = xrows;
   c->args_x.sweep = 0;
   c->args_y = a;
   c->args_y.tiles = c->d_ty;
   c->args_y.ntiles = c->nty;
+  c->args_y.tile_w = ystep;
+  c->args_y.tile_h = c->tile_y;
   c->args_y.redo_off = 2;
   c->args_y.sweep = 1;
+  c->args_y.lanes_y = t64.lanes_y;
+  if (prec == FVNA_FP64) c->blocks_y = blocks_y_fp64(c->args_y, sms);
   // Strang: the step ends after the second x1 sweep, so never in the x2 sweep
   const bool strang = cfg->splitting == FVNA_SPLIT_STRANG;
   c->args_x.x_half = strang ? 1 : 0;

@@ -1,0 +1,518 @@
+// fvna_face64.cuh -- the binary64 interface solver, limited flux and cell
+// update shared by the 2D and 3D sweeps (arXiv 1311.3004, section 3.2, eqs.
+// fv-hr, fluc:m, fluc:p, limiter), for NT = 1 or 2 transverse momenta.
+//
+// Two forms of each, with the same results bit for bit (a zero's sign aside):
+//   *_general  every formula in the order of its definition on the binary64
+//              unit (the including units are compiled with -fmad=false);
+//   *_fast     the same roundings with fewer instructions on that unit:
+//              reciprocals, quotients, roots and the products of the solver
+//              and of the limiter's sums run in integer arithmetic
+//              (fvna_int64f.cuh), comparisons and powers of two as integer
+//              operations on the bit patterns.
+// What bounds these sweeps is the binary64 unit (16 cycles a warp instruction
+// per SM).  A cell of a 2D sweep sent it 214 instructions in general form, 8
+// of ten cycles of the sweep; the fast form sends 91, and its 2,200 integer
+// instructions run beside them.  Measured, x1 sweep of 2048 x 2048 cells: 2.06
+// ms before, 0.78 now; x2 sweep with the source 2.56 and 1.03.  Which products
+// go to the integer pipes was found by trying: all of them (67 left on the
+// unit) 0.81 ms, none 0.97, those of the solver and the limiter's sums 0.78.
+//
+// Exact shortcuts of the fast form: halves are moved through products and
+// sums, which is exact while nothing is subnormal (S = 2 Z: u = S rcp(S1),
+// 2 Z2 = S2, Phi = 1 + (beta2/2)(S1 - 2), flux sums G = 2 F with dt/dx
+// halved instead); s1 W2 = W2 s1 is the product the wave already holds; a sum
+// is the fused multiply-add x 1 + y and a product x y + (-0), which round
+// once like the plain ones and are taken 16 % faster (16.1 against 19.1
+// cycles, measured).
+//
+// The fast form needs "tame" data: q1 within 1/16 of 1, momenta zero or of
+// magnitude [2^-170, 2^-4), |beta2| zero or [2^-40, 8], dt/dx in [2^-40, 2).
+// Then c is in (0.69, 1.3), every interface is subsonic, and following the
+// smallest nonzero values through (a difference of two numbers is zero or at
+// least a unit in the last place of the smaller): z 2^-171, their sums and u
+// 2^-226, r13 2^-229, a1 and a2 2^-224, W transverse 2^-453, a3 2^-506.  So
+// all factors of a product are zero or have exponent fields that add up to
+// 1034 or more, which is what mulz asks for, and no product or sum is
+// subnormal.  A limiter value below 2^-100 (but not zero) could make G
+// subnormal: the update then takes the general form.
+#pragma once
+
+#include "fvna_int64f.cuh"
+
+namespace fvna {
+namespace f64 {
+
+using int64f::hi_of;
+using int64f::mulz;
+
+enum { F64_MC = 0, F64_NONE = 1, F64_LW = 2 };   // the limiter kinds
+
+// 1.0 and -0.0, read from memory so that the compiler cannot see them and
+// turn the fused forms back into adds and multiplies
+static __device__ double g_unit[2] = {1.0, -0.0};
+struct Unit {
+  double one, nz;
+  __device__ __forceinline__ void load() {
+    one = *(volatile double *)&g_unit[0];
+    nz = *(volatile double *)&g_unit[1];
+  }
+  __device__ __forceinline__ double add(double x, double y) const { return __fma_rn(x, one, y); }
+  __device__ __forceinline__ double sub(double x, double y) const { return __fma_rn(x, one, -y); }
+  __device__ __forceinline__ double mul(double x, double y) const { return __fma_rn(x, y, nz); }
+};
+
+// Constants of a sweep.
+struct Par {
+  Unit U;
+  double beta2, bh, lam, hlam;   // 2 (beta - 1), half of it, dt/dx, half of it
+  bool ok;                       // the constants allow the fast form
+  __device__ __forceinline__ void set(double beta2_, double lam_) {
+    U.load();
+    beta2 = beta2_;
+    bh = 0.5 * beta2_;
+    lam = lam_;
+    hlam = 0.5 * lam_;
+    const double b = fabs(beta2_);
+    ok = (b == 0.0 || (b >= 0x1p-40 && b <= 8.0)) && lam_ >= 0x1p-40 && lam_ < 2.0;
+  }
+};
+
+// zero, or magnitude in [2^-170, 2^-4)
+__device__ __forceinline__ bool tame_momentum(double b) {
+  const unsigned h = hi_of(b) & 0x7fffffffu;
+  return h - 0x35500000u < 0x3fb00000u - 0x35500000u || (int64f::bits_of(b) << 1) == 0;
+}
+template <int NT> __device__ __forceinline__ bool tame_cell(const double q[2 + NT]) {
+  bool t = hi_of(q[0]) - 0x3fee0000u < 0x3ff10000u - 0x3fee0000u;   // [15/16, 17/16)
+#pragma unroll
+  for (int k = 1; k < 2 + NT; k++) t = t && tame_momentum(q[k]);
+  return t;
+}
+
+// One interface: speeds, and the waves of the two acoustic families
+// (a, a s, a r_k) and of the transverse ones (one component each).
+template <int NT> struct Face {
+  double s0, s1, u;
+  double a1, w01, w0[NT];
+  double a2, w11, w1[NT];
+  double w2[NT];
+};
+// Flux data of an interface; G is twice the correction flux of eq. limiter.
+template <int NT> struct Flux {
+  double am[2 + NT], ap[2 + NT], G[2 + NT];
+};
+
+// velocities z = (normal, transverse) / q1
+template <int NT>
+__device__ __forceinline__ void z_general(const double q[2 + NT], double z[1 + NT]) {
+  const double r = 1.0 / q[0];
+#pragma unroll
+  for (int k = 0; k < 1 + NT; k++) z[k] = q[1 + k] * r;
+}
+template <int NT> __device__ __forceinline__ void z_fast(const Par &P, const double q[2 + NT], double z[1 + NT]) {
+  const double r = int64f::rcp_mid(q[0]);
+#pragma unroll
+  for (int k = 0; k < 1 + NT; k++) z[k] = P.U.mul(q[1 + k], r);
+}
+
+// Roe solver (section 3.2) of cells L and R; true if the radicand is negative.
+template <int NT>
+__device__ __forceinline__ bool face_general(double beta2, const double L[2 + NT],
+                                             const double zL[1 + NT], const double R[2 + NT],
+                                             const double zR[1 + NT], Face<NT> &F) {
+  const double Z1 = 0.5 * (L[0] + R[0]);
+  const double Z2 = 0.5 * (zL[0] + zR[0]);
+  const double Phi = 1.0 + beta2 * (Z1 - 1.0);
+  const double rZ1 = 1.0 / Z1;
+  const double u = Z2 * rZ1;
+  const double D = u * u - 2.0 * Z2 * u + Phi;
+  const bool nonreal = D < 0.0;
+  const double c = sqrt(D);
+  F.s0 = u + c;
+  F.s1 = u - c;
+  F.u = u;
+  const double rc = 1.0 / c;
+  const double h = 0.5 * rc;
+  const double d1 = R[0] - L[0];
+  const double d2 = R[1] - L[1];
+  F.a1 = (d2 - F.s1 * d1) * h;
+  F.a2 = (F.s0 * d1 - d2) * h;
+  F.w01 = F.a1 * F.s0;
+  F.w11 = F.a2 * F.s1;
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    const double v = (0.5 * (zL[1 + k] + zR[1 + k])) * rZ1;
+    const double r1 = v * (F.s0 - 2.0 * Z2) * rc;
+    const double r2 = v * (2.0 * Z2 - F.s1) * rc;
+    F.w0[k] = F.a1 * r1;
+    F.w1[k] = F.a2 * r2;
+    F.w2[k] = (R[2 + k] - L[2 + k]) - F.w0[k] - F.w1[k];
+  }
+  return nonreal;
+}
+
+template <int NT>
+__device__ __forceinline__ void face_fast(const Par &P, const double L[2 + NT],
+                                          const double zL[1 + NT], const double R[2 + NT],
+                                          const double zR[1 + NT], Face<NT> &F) {
+  const Unit &U = P.U;
+  const double S1 = U.add(L[0], R[0]);
+  const double S2 = U.add(zL[0], zR[0]);
+  const double Phi = U.add(mulz(P.bh, U.add(S1, -2.0)), 1.0);
+  const double rs = int64f::rcp_mid(S1);
+  const double u = mulz(S2, rs);
+  const double D = U.add(U.sub(mulz(u, u), mulz(S2, u)), Phi);
+  const double c = int64f::sqrt_mid(D);
+  F.s0 = U.add(u, c);
+  F.s1 = U.sub(u, c);
+  F.u = u;
+  const double rc = int64f::rcp_mid(c);
+  const double h = int64f::half_of(rc);
+  const double d1 = U.sub(R[0], L[0]);
+  const double d2 = U.sub(R[1], L[1]);
+  const double e0 = U.sub(F.s0, S2), e1 = U.sub(S2, F.s1);
+  F.a1 = mulz(U.sub(d2, mulz(F.s1, d1)), h);
+  F.a2 = mulz(U.sub(mulz(F.s0, d1), d2), h);
+  F.w01 = mulz(F.a1, F.s0);
+  F.w11 = mulz(F.a2, F.s1);
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    const double v = mulz(U.add(zL[1 + k], zR[1 + k]), rs);
+    const double r1 = mulz(mulz(v, e0), rc);
+    const double r2 = mulz(mulz(v, e1), rc);
+    F.w0[k] = mulz(F.a1, r1);
+    F.w1[k] = mulz(F.a2, r2);
+    F.w2[k] = U.sub(U.sub(U.sub(R[2 + k], L[2 + k]), F.w0[k]), F.w1[k]);
+  }
+}
+
+// Limiter value for the ratio num/den of eq. limiter, 0 for a zero wave.
+template <int LIM> __device__ __forceinline__ double phi_general(double num, double den) {
+  if (LIM == F64_NONE) return 0.0;
+  if (LIM == F64_LW) return den > 0.0 ? 1.0 : 0.0;
+  const double theta = num / den;
+  const double a = 0.5 * (1.0 + theta);
+  double m = a < 2.0 ? a : 2.0;
+  const double b = 2.0 * theta;
+  m = m < b ? m : b;
+  m = m > 0.0 ? m : 0.0;
+  return den > 0.0 ? m : 0.0;
+}
+// den >= 0.  theta >= 3 gives 2, theta <= 0 gives 0; between, the smaller of
+// (1 + theta)/2 and 2 theta, compared as bit patterns.
+template <int LIM>
+__device__ __forceinline__ double phi_fast(const Unit &U, double num, double den, bool &tiny) {
+  if (LIM == F64_NONE) return 0.0;
+  if (LIM == F64_LW) return int64f::bits_of(den) ? 1.0 : 0.0;
+  int64f::u64 nb = int64f::bits_of(num), db = int64f::bits_of(den);
+  const bool on = (int64f::i64)nb > 0 && db != 0;
+  nb = on ? nb : 0x3ff0000000000000ull;
+  db = on ? db : 0x3ff0000000000000ull;
+  double theta;
+  if (int64f::mid((int64f::u32)(nb >> 32)) && int64f::mid((int64f::u32)(db >> 32)))
+    theta = int64f::div_mid(nb, db);
+  else
+    theta = int64f::of_bits(nb) / int64f::of_bits(db);
+  const int64f::u64 a = int64f::bits_of(int64f::half_of(U.add(theta, 1.0)));
+  const int64f::u64 b = int64f::bits_of(theta) + 0x10000000000000ull;
+  int64f::u64 m = a < b ? a : b;
+  m = hi_of(theta) >= 0x40080000u ? 0x4000000000000000ull : m;
+  m = on ? m : 0;
+  tiny |= on && (int64f::u32)(m >> 32) < (923u << 20);
+  return int64f::of_bits(m);
+}
+
+// Fluctuations and correction flux of face I between the faces Lf and Rf.
+template <int LIM, int NT>
+__device__ __forceinline__ void flux_general(const Face<NT> &I, const Face<NT> &Lf,
+                                             const Face<NT> &Rf, double lam, Flux<NT> &o) {
+  const double s0 = I.s0, s1 = I.s1, u = I.u;
+  const double sm0 = s0 < 0.0 ? s0 : 0.0, sp0 = s0 > 0.0 ? s0 : 0.0;
+  const double sm1 = s1 < 0.0 ? s1 : 0.0, sp1 = s1 > 0.0 ? s1 : 0.0;
+  const double smu = u < 0.0 ? u : 0.0, spu = u > 0.0 ? u : 0.0;
+  const bool l0 = s0 > 0.0, l1 = s1 > 0.0, lu = u > 0.0;
+  o.am[0] = sm0 * I.a1 + sm1 * I.a2;
+  o.ap[0] = sp0 * I.a1 + sp1 * I.a2;
+  o.am[1] = sm0 * I.w01 + sm1 * I.w11;
+  o.ap[1] = sp0 * I.w01 + sp1 * I.w11;
+  double d0 = I.a1 * I.a1 + I.w01 * I.w01;
+  double n0 = (l0 ? Lf.a1 : Rf.a1) * I.a1 + (l0 ? Lf.w01 : Rf.w01) * I.w01;
+  double d1 = I.a2 * I.a2 + I.w11 * I.w11;
+  double n1 = (l1 ? Lf.a2 : Rf.a2) * I.a2 + (l1 ? Lf.w11 : Rf.w11) * I.w11;
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    o.am[2 + k] = sm0 * I.w0[k] + sm1 * I.w1[k] + smu * I.w2[k];
+    o.ap[2 + k] = sp0 * I.w0[k] + sp1 * I.w1[k] + spu * I.w2[k];
+    d0 = d0 + I.w0[k] * I.w0[k];
+    n0 = n0 + (l0 ? Lf.w0[k] : Rf.w0[k]) * I.w0[k];
+    d1 = d1 + I.w1[k] * I.w1[k];
+    n1 = n1 + (l1 ? Lf.w1[k] : Rf.w1[k]) * I.w1[k];
+  }
+  const double as0 = fabs(s0), as1 = fabs(s1), asu = fabs(u);
+  const double c0 = as0 * (1.0 - lam * as0) * phi_general<LIM>(n0, d0);
+  const double c1 = as1 * (1.0 - lam * as1) * phi_general<LIM>(n1, d1);
+  o.G[0] = c0 * I.a1 + c1 * I.a2;
+  o.G[1] = c0 * I.w01 + c1 * I.w11;
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    const double U = lu ? Lf.w2[k] : Rf.w2[k];
+    const double c2 = asu * (1.0 - lam * asu) * phi_general<LIM>(U * I.w2[k], I.w2[k] * I.w2[k]);
+    o.G[2 + k] = c0 * I.w0[k] + c1 * I.w1[k] + c2 * I.w2[k];
+  }
+}
+
+// tiny: a limiter value was met with which G may be subnormal
+template <int LIM, int NT>
+__device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const Face<NT> &Lf,
+                                          const Face<NT> &Rf, Flux<NT> &o, bool &tiny) {
+  const Unit &U = P.U;
+  const bool neg = (int)hi_of(I.u) < 0;
+  o.am[0] = I.w11;
+  o.ap[0] = I.w01;
+  o.am[1] = U.mul(I.s1, I.w11);
+  o.ap[1] = U.mul(I.s0, I.w01);
+  double d0 = U.add(mulz(I.a1, I.a1), mulz(I.w01, I.w01));
+  double n0 = U.add(mulz(Lf.a1, I.a1), mulz(Lf.w01, I.w01));
+  double d1 = U.add(mulz(I.a2, I.a2), mulz(I.w11, I.w11));
+  double n1 = U.add(mulz(Rf.a2, I.a2), mulz(Rf.w11, I.w11));
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    // the transverse wave joins the fluctuation of the side it moves to
+    const double X = U.mul(I.s1, I.w1[k]), Y = U.mul(I.s0, I.w0[k]);
+    const double t = U.add(neg ? X : Y, U.mul(I.u, I.w2[k]));
+    o.am[2 + k] = neg ? t : X;
+    o.ap[2 + k] = neg ? Y : t;
+    d0 = U.add(d0, mulz(I.w0[k], I.w0[k]));
+    n0 = U.add(n0, mulz(Lf.w0[k], I.w0[k]));
+    d1 = U.add(d1, mulz(I.w1[k], I.w1[k]));
+    n1 = U.add(n1, mulz(Rf.w1[k], I.w1[k]));
+  }
+  const double as1 = -I.s1, asu = fabs(I.u);
+  const double c0 = U.mul(U.mul(I.s0, U.sub(1.0, U.mul(P.lam, I.s0))), phi_fast<LIM>(U, n0, d0, tiny));
+  const double c1 = U.mul(U.mul(as1, U.sub(1.0, U.mul(P.lam, as1))), phi_fast<LIM>(U, n1, d1, tiny));
+  const double fu = U.mul(asu, U.sub(1.0, U.mul(P.lam, asu)));
+  o.G[0] = U.add(U.mul(c0, I.a1), U.mul(c1, I.a2));
+  o.G[1] = U.add(U.mul(c0, I.w01), U.mul(c1, I.w11));
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    const double w = neg ? Rf.w2[k] : Lf.w2[k];
+    const double c2 =
+        U.mul(fu, phi_fast<LIM>(U, mulz(w, I.w2[k]), mulz(I.w2[k], I.w2[k]), tiny));
+    o.G[2 + k] = U.add(U.add(U.mul(c0, I.w0[k]), U.mul(c1, I.w1[k])), U.mul(c2, I.w2[k]));
+  }
+}
+
+// Cell update of eq. fv-hr.
+template <int NT>
+__device__ __forceinline__ void update_general(double lam, const double q[2 + NT], const double am[],
+                                               const double Gr[], const double ap[],
+                                               const double Gl[], double o[2 + NT]) {
+#pragma unroll
+  for (int k = 0; k < 2 + NT; k++)
+    o[k] = q[k] - lam * (am[k] + ap[k]) - lam * (0.5 * Gr[k] - 0.5 * Gl[k]);
+}
+template <int NT>
+__device__ __forceinline__ void update_fast(const Par &P, const double q[2 + NT], const double am[],
+                                            const double Gr[], const double ap[],
+                                            const double Gl[], double o[2 + NT]) {
+  const Unit &U = P.U;
+#pragma unroll
+  for (int k = 0; k < 2 + NT; k++)
+    o[k] = U.sub(U.sub(q[k], U.mul(P.lam, U.add(am[k], ap[k]))),
+                 mulz(P.hlam, U.sub(Gr[k], Gl[k])));
+}
+
+// max|s| as a bit pattern (|s3| = |u| never exceeds the other two)
+template <int NT>
+__device__ __forceinline__ void speed_max(unsigned long long &m, const Face<NT> &F) {
+  const unsigned long long b0 = int64f::bits_of(F.s0) & 0x7fffffffffffffffull,
+                           b1 = int64f::bits_of(F.s1) & 0x7fffffffffffffffull;
+  m = b0 > m ? b0 : m;
+  m = b1 > m ? b1 : m;
+}
+
+// ---------------------------------------------------------------------------
+// A segment of a line across the lanes: lane l holds the CPL consecutive
+// cells q[0..CPL-1], lane l + 1 the next ones.  Each lane solves the faces on
+// the left of its cells; neighbour cells, faces and fluxes come by shuffles.
+// On return o[] is the update of every cell that has two cells of the segment
+// on each side.  g = line coordinate of q[0], n = cells of the line: max|s|
+// is taken over the faces of the domain cells, the non-real test over the
+// extended line's, as the reference evaluation does.  Faces flo..fhi (face f
+// lies on the left of cell f) take no correction.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ double down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+template <int LIM, int NT, int CPL, bool FAST>
+__device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2 + NT], int g, int n,
+                                             unsigned long long &smax, bool &nonreal,
+                                             double o[CPL][2 + NT], int flo, int fhi) {
+  const int lane = threadIdx.x & 31;
+  double z[CPL][1 + NT], ql[2 + NT], zl[1 + NT];
+#pragma unroll
+  for (int i = 0; i < CPL; i++) {
+    if (FAST) z_fast<NT>(P, q[i], z[i]);
+    else z_general<NT>(q[i], z[i]);
+  }
+#pragma unroll
+  for (int k = 0; k < 2 + NT; k++) ql[k] = up1(q[CPL - 1][k]);
+#pragma unroll
+  for (int k = 0; k < 1 + NT; k++) zl[k] = up1(z[CPL - 1][k]);
+  Face<NT> F[CPL];
+#pragma unroll
+  for (int i = 0; i < CPL; i++) {
+    const double *L = i ? q[i ? i - 1 : 0] : ql, *zL = i ? z[i ? i - 1 : 0] : zl;
+    bool nr = false;
+    if (FAST) face_fast<NT>(P, L, zL, q[i], z[i], F[i]);
+    else nr = face_general<NT>(P.beta2, L, zL, q[i], z[i], F[i]);
+    const int gl = g + i - 1;                      // left cell of the face
+    if (i > 0 || lane > 0) {
+      if (!FAST && gl >= -2 && gl <= n) nonreal |= nr;
+      if (gl >= -1 && gl <= n - 1) speed_max(smax, F[i]);
+    }
+  }
+  // the face before this lane's first one, and the one after its last
+  Face<NT> A, B;
+  A.a1 = up1(F[CPL - 1].a1); A.w01 = up1(F[CPL - 1].w01);
+  B.a2 = down1(F[0].a2); B.w11 = down1(F[0].w11);
+  if (!FAST) {
+    A.a2 = up1(F[CPL - 1].a2); A.w11 = up1(F[CPL - 1].w11);
+    B.a1 = down1(F[0].a1); B.w01 = down1(F[0].w01);
+  }
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    A.w0[k] = up1(F[CPL - 1].w0[k]); A.w2[k] = up1(F[CPL - 1].w2[k]);
+    B.w1[k] = down1(F[0].w1[k]); B.w2[k] = down1(F[0].w2[k]);
+    if (!FAST) {
+      A.w1[k] = up1(F[CPL - 1].w1[k]);
+      B.w0[k] = down1(F[0].w0[k]);
+    }
+  }
+  Flux<NT> X[CPL];
+  bool tiny = false;
+#pragma unroll
+  for (int i = 0; i < CPL; i++) {
+    const Face<NT> &Lf = i ? F[i ? i - 1 : 0] : A, &Rf = i + 1 < CPL ? F[i + 1 < CPL ? i + 1 : 0] : B;
+    if (FAST) flux_fast<LIM, NT>(P, F[i], Lf, Rf, X[i], tiny);
+    else flux_general<LIM, NT>(F[i], Lf, Rf, P.lam, X[i]);
+    if (g + i >= flo && g + i <= fhi) {
+#pragma unroll
+      for (int k = 0; k < 2 + NT; k++) X[i].G[k] = 0.0;
+    }
+  }
+  const bool half = FAST && !__any_sync(0xffffffffu, tiny);
+  double am[2 + NT], G[2 + NT];                    // the next lane's first face
+#pragma unroll
+  for (int k = 0; k < 2 + NT; k++) {
+    am[k] = down1(X[0].am[k]);
+    G[k] = down1(X[0].G[k]);
+  }
+#pragma unroll
+  for (int i = 0; i < CPL; i++) {
+    const double *mr = i + 1 < CPL ? X[i + 1 < CPL ? i + 1 : 0].am : am;
+    const double *Gr = i + 1 < CPL ? X[i + 1 < CPL ? i + 1 : 0].G : G;
+    if (half) update_fast<NT>(P, q[i], mr, Gr, X[i].ap, X[i].G, o[i]);
+    else update_general<NT>(P.lam, q[i], mr, Gr, X[i].ap, X[i].G, o[i]);
+  }
+}
+
+// The segment in the form its data allow.
+template <int LIM, int NT, int CPL>
+__device__ __forceinline__ void lanes_step(const Par &P, const double q[CPL][2 + NT], int g, int n,
+                                           unsigned long long &smax, bool &nonreal,
+                                           double o[CPL][2 + NT], int flo = 1, int fhi = 0) {
+  bool t = P.ok;
+#pragma unroll
+  for (int i = 0; i < CPL; i++) t = t && tame_cell<NT>(q[i]);
+  if (__all_sync(0xffffffffu, t)) lanes_update<LIM, NT, CPL, true>(P, q, g, n, smax, nonreal, o, flo, fhi);
+  else lanes_update<LIM, NT, CPL, false>(P, q, g, n, smax, nonreal, o, flo, fhi);
+}
+
+// ---------------------------------------------------------------------------
+// A line marched by each lane: cells are pushed in order, j = 0, 1, ...; face
+// j lies between cells j - 1 and j.  From j = 4 on a push returns the update
+// of cell j - 2.  Called by all lanes of the warp together.
+// ---------------------------------------------------------------------------
+template <int LIM, int NT> struct March {
+  double c1[2 + NT], c2[2 + NT], z1[1 + NT];
+  Face<NT> f1, f2;            // faces j - 1 and j - 2
+  double ap[2 + NT], G[2 + NT];
+  int run;                    // tame cells in a row, the same in all lanes
+  bool lhalf;                 // the left face's G may be halved after the fact
+  unsigned long long smax;
+  bool nonreal;
+
+  __device__ __forceinline__ void init() {
+    run = 0;
+    lhalf = true;
+    smax = 0;
+    nonreal = false;
+  }
+  // count_speed: face j - 1 counts towards max|s|; count_real: face j towards
+  // the non-real test; plain: no correction on face j - 1
+  __device__ __forceinline__ bool push(const Par &P, int j, const double q[2 + NT],
+                                       double out[2 + NT], bool count_speed, bool count_real,
+                                       bool plain) {
+    run = __all_sync(0xffffffffu, P.ok && tame_cell<NT>(q)) ? run + 1 : 0;
+    // this cell and the four before it
+    if (run > (j < 4 ? j : 4)) step<true>(P, j, q, out, count_speed, count_real, plain);
+    else step<false>(P, j, q, out, count_speed, count_real, plain);
+    return j >= 4;
+  }
+  template <bool FAST>
+  __device__ __forceinline__ void step(const Par &P, int j, const double q[2 + NT],
+                                       double out[2 + NT], bool count_speed, bool count_real,
+                                       bool plain) {
+    double z[1 + NT];
+    if (FAST) z_fast<NT>(P, q, z);
+    else z_general<NT>(q, z);
+    if (j > 0) {
+      Face<NT> f;
+      if (FAST) face_fast<NT>(P, c1, z1, q, z, f);
+      else {
+        const bool nr = face_general<NT>(P.beta2, c1, z1, q, z, f);
+        if (count_real) nonreal |= nr;
+      }
+      if (j >= 3) {
+        Flux<NT> X;
+        bool half = FAST;
+        if (FAST) {
+          bool tiny = false;
+          flux_fast<LIM, NT>(P, f1, f2, f, X, tiny);
+          half = !__any_sync(0xffffffffu, tiny);
+        } else {
+          flux_general<LIM, NT>(f1, f2, f, P.lam, X);
+        }
+        if (plain) {
+#pragma unroll
+          for (int k = 0; k < 2 + NT; k++) X.G[k] = 0.0;
+        }
+        if (count_speed) speed_max(smax, f1);
+        if (j >= 4) {
+          if (half && lhalf) update_fast<NT>(P, c2, X.am, X.G, ap, G, out);
+          else update_general<NT>(P.lam, c2, X.am, X.G, ap, G, out);
+        }
+#pragma unroll
+        for (int k = 0; k < 2 + NT; k++) {
+          ap[k] = X.ap[k];
+          G[k] = X.G[k];
+        }
+        lhalf = half;
+      }
+      f2 = f1;
+      f1 = f;
+    }
+#pragma unroll
+    for (int k = 0; k < 2 + NT; k++) {
+      c2[k] = c1[k];
+      c1[k] = q[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 1 + NT; k++) z1[k] = z[k];
+  }
+};
+
+}  // namespace f64
+}  // namespace fvna

@@ -15,8 +15,6 @@
 
 #define POLICY P32
 #define SUFFIX fp32
-#define HAS_COMP 1
-#define FVNA_PRECISION_SWEEPS 0
 #include "fvna_precision.inc"
 
 namespace fvna {

@@ -7,15 +7,162 @@
 // number of the previous step).
 #include "fvna_launch.h"
 #include "fvna_step.cuh"
-#include "fvna_sweeps.cuh"
+#include "fvna_sweeps64.cuh"
 
 #define POLICY P64
 #define SUFFIX fp64
-#define HAS_COMP 0
-#define FVNA_PRECISION_SWEEPS 1
 #include "fvna_precision.inc"
 
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
 namespace fvna {
+
+namespace {
+
+typedef void (*StepKernel)(StepArgs);
+
+constexpr size_t SMEM_Y64 = (size_t)WARPS_PER_BLOCK * YRING * 96 * sizeof(double);
+
+template <int CPL> StepKernel px(int lim) {
+  return lim == LIM_NONE ? k_sweep_x64<CPL, LIM_NONE>
+         : lim == LIM_LW ? k_sweep_x64<CPL, LIM_LW>
+                         : k_sweep_x64<CPL, LIM_MC>;
+}
+StepKernel pick_x(int tile_x, int lim) { return tile_x == 64 ? px<2>(lim) : px<1>(lim); }
+StepKernel pick_y(int lim) {
+  return lim == LIM_NONE ? k_sweep_y64<YRING, LIM_NONE>
+         : lim == LIM_LW ? k_sweep_y64<YRING, LIM_LW>
+                         : k_sweep_y64<YRING, LIM_MC>;
+}
+
+}  // namespace
+
+int x64_cells(int tile_x) { return tile_x == 64 ? X64_OUT<2> : X64_OUT<1>; }
+
+static StepKernel pick_yl(int lim) {
+  return lim == LIM_NONE ? k_sweep_yl64<LIM_NONE>
+         : lim == LIM_LW ? k_sweep_yl64<LIM_LW>
+                         : k_sweep_yl64<LIM_MC>;
+}
+// shared memory of a tile of w columns with lanes along x2
+static size_t smem_yl(int w) { return (size_t)(w + 2) * 160 * sizeof(double); }
+
+cudaError_t prepare_kernels_fp64(int, int lim, int) {
+  return cudaFuncSetAttribute(pick_y(lim), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)SMEM_Y64);
+}
+static int occupancy(StepKernel k, size_t smem) {
+  int n = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, WARPS_PER_BLOCK * 32, smem);
+  return std::max(n, 1);
+}
+// Resident blocks of the sweeps per SM, asked for once per device and limiter.
+struct Occupancy64 {
+  int x1, x2, y, yl[8];      // yl[k - 1]: tiles of 4 k - 2 columns
+};
+static Occupancy64 occupancy64(int lim) {
+  constexpr int DEVICES = 64;
+  static std::mutex m;
+  static bool known[DEVICES][3];
+  static Occupancy64 kept[DEVICES][3];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(m);
+  const bool keep = dev >= 0 && dev < DEVICES && lim >= 0 && lim < 3;
+  if (keep && known[dev][lim]) return kept[dev][lim];
+  Occupancy64 o;
+  o.x1 = occupancy(pick_x(32, lim), 0);
+  o.x2 = occupancy(pick_x(64, lim), 0);
+  o.y = occupancy(pick_y(lim), SMEM_Y64);
+  for (int k = 1; k <= 8; k++) o.yl[k - 1] = occupancy(pick_yl(lim), smem_yl(4 * k - 2));
+  if (keep) {
+    kept[dev][lim] = o;
+    known[dev][lim] = true;
+  }
+  return o;
+}
+int occupancy_x_fp64(int tile_x, int lim, int) {
+  const Occupancy64 o = occupancy64(lim);
+  return tile_x == 64 ? o.x2 : o.x1;
+}
+int occupancy_y_fp64(int lim, int) { return occupancy64(lim).y; }
+cudaError_t launch_sweep_x_fp64(int tile_x, const StepArgs &a, int blocks, cudaStream_t s) {
+  pick_x(tile_x, a.limiter)<<<blocks, WARPS_PER_BLOCK * 32, 0, s>>>(a);
+  return cudaGetLastError();
+}
+cudaError_t launch_sweep_y_fp64(const StepArgs &a, int blocks, cudaStream_t s) {
+  if (a.lanes_y)
+    pick_yl(a.limiter)<<<blocks, WARPS_PER_BLOCK * 32, smem_yl(a.tile_w), s>>>(a);
+  else
+    pick_y(a.limiter)<<<blocks, WARPS_PER_BLOCK * 32, SMEM_Y64, s>>>(a);
+  return cudaGetLastError();
+}
+int blocks_y_fp64(const StepArgs &a, int sms) {
+  if (a.lanes_y) return std::min(a.ntiles, occupancy64(a.limiter).yl[(a.tile_w + 2) / 4 - 1] * sms);
+  return std::min((a.ntiles + WARPS_PER_BLOCK - 1) / WARPS_PER_BLOCK,
+                  occupancy_y_fp64(a.limiter, 0) * sms);
+}
+
+// Tile shapes of the binary64 sweeps.  The binary64 unit of an SM quarter is
+// what a sweep waits for, so its time is that of the quarter with the most
+// cells to do.  Tiles are dealt to the resident warps (blocks) in turn, so a
+// quarter with r of them does r tiles per full round and the rest of the last
+// round; a warp alone on its quarter cannot use its two pipes side by side and
+// counts as ALONE warps.  The x2 sweep marches tall tiles where there are
+// cells enough for them, and takes the lanes along x2 otherwise (26 of 32
+// lanes useful, but a column is a unit of work).
+void pick_tiles64(int n, const Extent *d, int sms, int lim, int tile_x, int tile_y, Tiles64 *t) {
+  constexpr double ALONE = 2.2;
+  auto load = [&](double tiles, int r, double slots) {
+    const double rounds = std::floor(tiles / (r * slots));
+    return std::max(rounds * r + std::ceil((tiles - rounds * r * slots) / slots), ALONE);
+  };
+  auto tiles = [&](int w, int h) {
+    double c = 0;
+    for (int k = 0; k < n; k++)
+      c += (double)((d[k].nx + w - 1) / w) * ((d[k].ny + h - 1) / h);
+    return c;
+  };
+  const Occupancy64 o = occupancy64(lim);
+  const double quarters = 4.0 * sms;
+  double best = 1e300;
+  for (int tx : {64, 32}) {
+    if (tile_x && (tile_x == 64) != (tx == 64)) continue;
+    const double items = tiles(x64_cells(tx), 1);
+    const double c = load(items, tx == 64 ? o.x2 : o.x1, quarters) * (tx == 64 ? 2.4 : 1);
+    if (c < best) {
+      best = c;
+      t->tile_x = tile_x ? tile_x : tx;
+      t->rows_x = (int)std::min(8.0, std::max(1.0, items / (64.0 * quarters)));
+    }
+  }
+  t->lanes_y = 0;
+  t->w_y = YCOLS;
+  t->tile_y = tile_y;
+  if (tile_y) return;
+  best = 1e300;
+  int most = 1;
+  for (int k = 0; k < n; k++) most = std::max(most, d[k].ny);
+  for (int ty = 1; ty <= std::min(most, 256); ty++) {
+    const double c = load(tiles(YCOLS, ty), o.y, quarters) * (ty + 2 * HALO_Y);
+    if (c < best) {
+      best = c;
+      t->tile_y = ty;
+    }
+  }
+  for (int k = 1; k <= 8; k++) {
+    const int w = 4 * k - 2;
+    const double c = load(tiles(w, YL_ROWS), o.yl[k - 1], sms) * k;
+    if (c < best) {
+      best = c;
+      t->lanes_y = 1;
+      t->w_y = w;
+      t->tile_y = YL_ROWS;
+    }
+  }
+}
 
 // End of a step for every domain (see fvna_step.cuh).
 __global__ void k_advance(StepArgs A) {

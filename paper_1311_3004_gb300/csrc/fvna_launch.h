@@ -10,9 +10,6 @@ namespace fvna {
 constexpr int WARPS_PER_BLOCK = 4;
 constexpr int YRING = 8;  // rows in flight per warp in the x2 sweep
 
-// shared memory of one block of each sweep (bytes)
-size_t smem_sweep_x(int precision, int tile_x);
-size_t smem_sweep_y(int precision);
 // one-time attribute setup (opt-in shared memory); returns cudaSuccess or the error
 cudaError_t prepare_kernels(int precision, int tile_x, int lim, int comp);
 // resident blocks per SM of each sweep
@@ -56,6 +53,8 @@ cudaError_t launch_riemann(int precision, double beta, int n, const double *qL, 
 // per-precision definitions (fvna_fp64.cu / fvna_fp32.cu)
 cudaError_t launch_sweep_x_fp64(int tile_x, const StepArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_sweep_y_fp64(const StepArgs &a, int blocks, cudaStream_t s);
+// blocks of the binary64 x2 sweep's persistent grid
+int blocks_y_fp64(const StepArgs &a, int sms);
 cudaError_t launch_speeds_fp64(const StepArgs &a, int dom, cudaStream_t s);
 cudaError_t launch_import_fp64(const DomDev &d, const double *q0, cudaStream_t s);
 cudaError_t launch_export_fp64(const DomDev &d, double *out, int what, cudaStream_t s);
@@ -75,6 +74,19 @@ cudaError_t launch_riemann_fp32(double beta, int n, const double *qL, const doub
 cudaError_t prepare_kernels_fp32(int tile_x, int lim, int comp);
 int occupancy_x_fp32(int tile_x, int lim, int comp);
 int occupancy_y_fp32(int lim, int comp);
+
+// binary64 sweeps: tile shapes for a set of domains (tile_x, tile_y: the
+// caller's, 0 = open), and the cells a segment of the x1 sweep updates
+struct Extent {
+  int nx, ny;
+};
+struct Tiles64 {
+  int tile_x, rows_x;           // x1 sweep: width choice, rows of a tile
+  int lanes_y, w_y, tile_y;     // x2 sweep: lanes along x2, columns and rows of a tile
+};
+void pick_tiles64(int n, const Extent *d, int sms, int lim, int tile_x, int tile_y,
+                  Tiles64 *t);
+int x64_cells(int tile_x);
 
 // binary32 sweeps (fvna_fp32.cu): x1 tiles are 32 rows x 2*x32_half(tile_x)
 // cells, x2 tiles 60 columns x tile_y rows; TMA tensor maps of every domain

@@ -29,6 +29,9 @@
 #include "fvna_sweeps.cuh"
 #include "fvna_x2.cuh"
 
+#define FVNA_PRAGMA(x) _Pragma(#x)
+#define FVNA_UNROLL(n) FVNA_PRAGMA(unroll n)
+
 namespace fvna {
 
 constexpr int X32_ROWS = 32;
@@ -844,7 +847,7 @@ __global__ void __launch_bounds__(32, Y32_MINBLOCKS) k_sweep_y32(StepArgs A) {
     // one code path for all tiles (border rules are per-row branches that
     // chunks away from the domain edges skip)
     // a tile's height: its own (the host may mix heights), else the sweep's
-    const int TY = tl.pad > 0 ? tl.pad : A.tile_y;
+    const int TY = tl.rows > 0 ? tl.rows : A.tile_y;
     int rc = REDO ? x2::y32_tile<LIM, COMP, false>(A, D, S, maps[tl.dom], ring, bars, used, x0,
                                                     y0, TY, lane)
                   : x2::y32_tile<LIM, COMP, true>(A, D, S, maps[tl.dom], ring, bars, used, x0, y0,

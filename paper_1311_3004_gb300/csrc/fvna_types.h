@@ -60,18 +60,21 @@ struct DomScal {
   double outflow[3];
 };
 
-// One warp's work item: domain, the tile origin (cells) and, for the
-// binary32 x2 sweep, the tile's height (0: the sweep's tile_y).
+// One warp's work item: domain, the tile origin (cells) and the tile's height
+// in rows (0 in the binary32 x2 sweep: the sweep's tile_y).
 struct Tile {
-  int dom, x0, y0, pad;
+  int dom, x0, y0, rows;
 };
 
 // Arguments of every step kernel.
 struct StepArgs {
   const DomDev *doms;
   DomScal *scal;
-  const Tile *tiles;
+  const Tile *tiles;             // NULL (binary64, one domain): tiles of tile_w x tile_h cells
+                                 // in row order
   int ntiles;
+  int tile_w, tile_h;
+  int lanes_y;                   // binary64 x2 sweep: 1 = lanes along x2 (k_sweep_yl64)
   int ndom;
   double beta, delta, dx, nu_w, nu_max, dt_fixed;
   int limiter, geometry, sweeps, tile_y;
