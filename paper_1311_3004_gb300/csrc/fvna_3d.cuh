@@ -17,6 +17,7 @@
 // at u, eigenvectors r1, r2 with fourth components w (s1 - 2 Z2)/c and
 // w (2 Z2 - s2)/c, w = Z4/Z1).
 //
+// binary32 sweeps (the binary64 one is in fvna_3d_sweep64.cuh):
 //   k3_sweep_x   x1 sweep: a warp holds 64 cells of one row, two per lane,
 //                each lane solving the faces on the left of its cells and
 //                exchanging neighbour faces by shuffles; 60 cells updated
@@ -25,11 +26,14 @@
 //                march together along x2 (or x3) over TY cells plus two halo
 //                cells at each end, loading and storing one coalesced row per
 //                field and cell.
+// both precisions:
 //   k3_source    forward Euler with the 7-point Laplacian of z = q/q1.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "fvna_int64f.cuh"
 
 namespace fvna {
 namespace d3 {
@@ -107,7 +111,10 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   return r;
 }
 
-__device__ __forceinline__ double inv_q1(double a) { return 1.0 / a; }
+// 1/x, correctly rounded (in integer arithmetic where x allows)
+__device__ __forceinline__ double inv_q1(double a) {
+  return int64f::mid(int64f::hi_of(a)) ? int64f::rcp_mid(a) : 1.0 / a;
+}
 __device__ __forceinline__ float inv_q1(float a) { return rcp_nr(1.0f + a); }
 
 // Roe solver of one interface, binary64, in the order of the definitions.
@@ -745,9 +752,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
           out[0][off] = qc[0];
 #pragma unroll
           for (int f = 0; f < 3; f++) {
-            T L = ((sz[f][ty + 1][tx] + sz[f][ty + 1][tx + 2]) +
-                   (sz[f][ty][tx + 1] + sz[f][ty + 2][tx + 1]) - T(4) * zc[f]) +
-                  ((zb[f] + zt[f]) - T(2) * zc[f]);
+            // 4 z and 2 z are exact: the fused forms round like the differences
+            T L = fma(T(-4), zc[f], (sz[f][ty + 1][tx] + sz[f][ty + 1][tx + 2]) +
+                                        (sz[f][ty][tx + 1] + sz[f][ty + 2][tx + 1])) +
+                  fma(T(-2), zc[f], zb[f] + zt[f]);
             out[1 + f][off] = qc[1 + f] + coef * L;
           }
         }

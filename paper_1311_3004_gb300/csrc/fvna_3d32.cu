@@ -5,5 +5,42 @@
 
 #define T3 float
 #define SFX 32
-#define HAS_COMP3 1
 #include "fvna_3d.inc"
+
+namespace fvna {
+namespace d3 {
+
+namespace {
+typedef void (*K3)(Args3);
+template <int LIM> K3 kx_c(bool comp) {
+  return comp ? k3_sweep_x<float, LIM, true> : k3_sweep_x<float, LIM, false>;
+}
+K3 kx(int lim, bool comp) {
+  return lim == L_NONE ? kx_c<L_NONE>(comp) : lim == L_LW ? kx_c<L_LW>(comp) : kx_c<L_MC>(comp);
+}
+template <int LIM> K3 kv_c(bool comp) {
+  return comp ? k3_sweep_v<float, LIM, true> : k3_sweep_v<float, LIM, false>;
+}
+K3 kv(int lim, bool comp) {
+  return lim == L_NONE ? kv_c<L_NONE>(comp) : lim == L_LW ? kv_c<L_LW>(comp) : kv_c<L_MC>(comp);
+}
+}  // namespace
+
+int tile_x3_32() { return X3_OUT; }
+
+// resident blocks per SM of the two sweep kernels
+void occupancy3_32(int lim, int comp, int *occ_x, int *occ_v) {
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ_x, kx(lim, comp != 0), 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ_v, kv(lim, comp != 0), 128, 0);
+}
+cudaError_t launch3_sweep_x_32(const Args3 &a, int blocks, cudaStream_t s) {
+  kx(a.limiter, a.comp != 0)<<<blocks, 128, 0, s>>>(a);
+  return cudaGetLastError();
+}
+cudaError_t launch3_sweep_v_32(const Args3 &a, int blocks, cudaStream_t s) {
+  kv(a.limiter, a.comp != 0)<<<blocks, 128, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace d3
+}  // namespace fvna

@@ -2,16 +2,35 @@
 // -fmad=false: every expression rounds as written, the order of the
 // definitions in fvna_3d.cuh), and the binary64 step bookkeeping of the 3D
 // contexts (both precisions).
-#include "fvna_3d.cuh"
+#include "fvna_3d_sweep64.cuh"
 #include "fvna_launch3.h"
+
+#include <algorithm>
 
 #define T3 double
 #define SFX 64
-#define HAS_COMP3 0
 #include "fvna_3d.inc"
 
 namespace fvna {
 namespace d3 {
+
+namespace {
+typedef void (*K3)(Args3);
+K3 k64(int lim) {
+  return lim == L_NONE ? k3_sweep64<L_NONE> : lim == L_LW ? k3_sweep64<L_LW> : k3_sweep64<L_MC>;
+}
+}  // namespace
+
+int occupancy3_64(int lim) {
+  int n = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k64(lim), 128, 0);
+  return std::max(n, 1);
+}
+cudaError_t launch3_sweep_64(const Args3 &a, int blocks, cudaStream_t s) {
+  const long long need = (segments64(a.d, a.dir) + 3) / 4;
+  k64(a.limiter)<<<(int)std::min<long long>(need, blocks), 128, 0, s>>>(a);
+  return cudaGetLastError();
+}
 
 __global__ void k3_first_dt(Args3 A, double dt0) {
   Scal3 *S = A.S;

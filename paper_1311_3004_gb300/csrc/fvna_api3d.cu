@@ -88,8 +88,8 @@ int enqueue_step(fvna3_ctx *c, cudaStream_t s, cudaEvent_t *ev) {
   for (int d = 0; d < 3; d++) {
     if (sw & (1 << d)) {
       Args3 a = with_planes(c, cur, nxt, d);
-      if (d == 0) CK3(fp64(c) ? launch3_sweep_x_64(a, c->blocks_x, s) : launch3_sweep_x_32(a, c->blocks_x, s));
-      else CK3(fp64(c) ? launch3_sweep_v_64(a, c->blocks_v, s) : launch3_sweep_v_32(a, c->blocks_v, s));
+      if (fp64(c)) CK3(launch3_sweep_64(a, c->blocks_x, s));
+      else CK3(d == 0 ? launch3_sweep_x_32(a, c->blocks_x, s) : launch3_sweep_v_32(a, c->blocks_v, s));
       std::swap(cur, nxt);
     }
     CK3(mark(1 + d));
@@ -242,9 +242,8 @@ int init3(const fvna_config *cfg, const fvna_domain3 *dom, const double *q0, int
   int dev = 0, sms = 0, ox = 0, ov = 0;
   CK3(cudaGetDevice(&dev));
   CK3(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  if (fp64(c)) occupancy3_64(cfg->limiter, 0, &ox, &ov);
-  else occupancy3_32(cfg->limiter, a.comp, &ox, &ov);
-  const int tx = fp64(c) ? tile_x3_64() : tile_x3_32();
+  if (!fp64(c)) occupancy3_32(cfg->limiter, a.comp, &ox, &ov);
+  const int tx = tile_x3_32();
   const long long xt = (long long)((D.nx + tx - 1) / tx) * D.ny * (long long)D.nz;
   const long long vt2 = (long long)((D.nx + 31) / 32) * ((D.ny + a.tile - 1) / a.tile) * D.nz;
   const long long vt3 = (long long)((D.nx + 31) / 32) * ((D.nz + a.tile - 1) / a.tile) * D.ny;
@@ -253,6 +252,7 @@ int init3(const fvna_config *cfg, const fvna_domain3 *dom, const double *q0, int
                                                                 (long long)std::max(ox, 1) * sms));
   c->blocks_v = (int)std::max<long long>(1, std::min<long long>((vt + 3) / 4,
                                                                 (long long)std::max(ov, 1) * sms));
+  if (fp64(c)) c->blocks_x = occupancy3_64(cfg->limiter) * sms;
   c->blocks_e = std::max(1, std::min((int)((D.plane + 255) / 256), 16 * sms));
   c->kernels_per_step = kernels_per_step(substeps(c));
 

@@ -8,13 +8,13 @@
 namespace fvna {
 namespace d3 {
 
-int tile_x3_64();
 int tile_x3_32();
-void occupancy3_64(int lim, int comp, int *occ_x, int *occ_v);
+// binary64: one sweep kernel (Args3::dir says which); resident blocks per SM,
+// and a launch of at most `blocks` blocks
+int occupancy3_64(int lim);
+cudaError_t launch3_sweep_64(const Args3 &a, int blocks, cudaStream_t s);
 void occupancy3_32(int lim, int comp, int *occ_x, int *occ_v);
-cudaError_t launch3_sweep_x_64(const Args3 &a, int blocks, cudaStream_t s);
 cudaError_t launch3_sweep_x_32(const Args3 &a, int blocks, cudaStream_t s);
-cudaError_t launch3_sweep_v_64(const Args3 &a, int blocks, cudaStream_t s);
 cudaError_t launch3_sweep_v_32(const Args3 &a, int blocks, cudaStream_t s);
 cudaError_t launch3_source_64(const Args3 &a, int blocks, cudaStream_t s);
 cudaError_t launch3_source_32(const Args3 &a, int blocks, cudaStream_t s);

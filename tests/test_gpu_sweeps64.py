@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from paper_1311_3004_gb300 import workloads as wl
-from tests.helpers import Case, run_gpu, run_oracle
+from helpers import Case, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -77,3 +77,19 @@ def test_states(name, limiter):
     qg, sg = run_gpu(c, steps)
     assert so["status"] == 0 and sg["rc"] == 0
     assert np.array_equal(qg, qo)
+
+
+@pytest.mark.parametrize("shape", [(28, 29, 57), (56, 27, 3), (1, 5, 30), (61, 2, 28)])
+@pytest.mark.parametrize("amp,thin", [(1e-3, 1.0), (1e-3, 1e-60), (0.08, 1.0)])
+def test_3d_edges(shape, amp, thin):
+    """Edges of the 28-cell segments along each axis, momenta below the fast
+    form's bounds, amplitudes beyond them."""
+    from test_gpu_3d import _run
+    nx, ny, nz = shape
+    q0 = wl.random_smooth3(nx, ny, nz, amp, seed=nx + nz)
+    q0[2] *= thin
+    q0[3, :, ny // 2:] = 0.0
+    q, st, qo, so = _run(nx, ny, nz, q0, (E, E, E, E, E, E) if 1 in shape or 2 in shape else
+                         (P, P, R, E, E, R), 5)
+    assert st["rc"] == 0 and so["status"] == 0
+    assert np.array_equal(q, qo)
