@@ -26,16 +26,29 @@
 // once like the plain ones and are taken 16 % faster (16.1 against 19.1
 // cycles, measured).
 //
-// The fast form needs "tame" data: q1 within 1/16 of 1, momenta zero or of
-// magnitude [2^-170, 2^-4), |beta2| zero or [2^-40, 8], dt/dx in [2^-40, 2).
-// Then c is in (0.69, 1.3), every interface is subsonic, and following the
-// smallest nonzero values through (a difference of two numbers is zero or at
-// least a unit in the last place of the smaller): z 2^-171, their sums and u
-// 2^-226, r13 2^-229, a1 and a2 2^-224, W transverse 2^-453, a3 2^-506.  So
-// all factors of a product are zero or have exponent fields that add up to
-// 1034 or more, which is what mulz asks for, and no product or sum is
-// subnormal.  A limiter value below 2^-100 (but not zero) could make G
-// subnormal: the update then takes the general form.
+// The fast form needs q1 within 1/16 of 1, momenta below 2^-4, |beta2| zero or
+// in [2^-40, 8] and dt/dx in [2^-40, 2): then c is in (0.69, 1.3) and every
+// interface is subsonic.  Integer products and the moved halves are used
+// (SOFT) while momenta are zero or at least 2^-400; with smaller ones the
+// products and halves are taken on the unit as defined (FAST).  Following the
+// smallest nonzero values through from there (a difference of two numbers is
+// zero or at least a unit in the last place of the smaller): z 2^-401, sums of
+// z and u 2^-455, r13 2^-458, a1 and a2 2^-454, w0 and w1 2^-912.  So every
+// factor pair given to mulz is zero or has exponent fields that add up to
+// 1034 or more, with two exceptions that do no harm: u u and S2 u, and the
+// transverse terms of the acoustic families' dot products, come out as zero
+// when they are below 2^-1012, where they are below 2^-54 of the sum they
+// join (1, and a1^2 or a1 U.a1, which is 2^-908 or more; the terms of
+// that sum have one sign).  The transverse family's own two products stay on
+// the unit.  A limiter value below 2^-100 or a transverse flux sum below
+// 2^-900 (but not zero) could make the halved sums subnormal: the update then
+// takes the general form.
+//
+// A pulse in a medium at rest sends a precursor of ever smaller momenta ahead
+// of itself, a cell a step, down to the subnormals.  One cell in a hundred
+// of the 2048^2 pulse is in it, but a marched tile that takes the general form
+// there is the slowest of its sweep: with that form below 2^-900 the x2 sweep
+// took 1.4 to 1.9 ms instead of 1.0.
 #pragma once
 
 #include "fvna_int64f.cuh"
@@ -78,16 +91,24 @@ struct Par {
   }
 };
 
-// zero, or magnitude in [2^-170, 2^-4)
-__device__ __forceinline__ bool tame_momentum(double b) {
-  const unsigned h = hi_of(b) & 0x7fffffffu;
-  return h - 0x35500000u < 0x3fb00000u - 0x35500000u || (int64f::bits_of(b) << 1) == 0;
-}
-template <int NT> __device__ __forceinline__ bool tame_cell(const double q[2 + NT]) {
-  bool t = hi_of(q[0]) - 0x3fee0000u < 0x3ff10000u - 0x3fee0000u;   // [15/16, 17/16)
+// The form a cell's values allow: GENERAL any, FAST, SOFT (see above).
+enum { GENERAL = 0, FAST = 1, SOFT = 2 };
+template <int NT> __device__ __forceinline__ int form_of(const double q[2 + NT]) {
+  unsigned lo = 0x3fa00000u, hi = 0;
 #pragma unroll
-  for (int k = 1; k < 2 + NT; k++) t = t && tame_momentum(q[k]);
-  return t;
+  for (int k = 1; k < 2 + NT; k++) {
+    const unsigned h = hi_of(q[k]) & 0x7fffffffu;
+    hi = h > hi ? h : hi;
+    lo = h < lo && (int64f::bits_of(q[k]) << 1) != 0 ? h : lo;
+  }
+  if (hi_of(q[0]) - 0x3fee0000u >= 0x3ff10000u - 0x3fee0000u || hi >= 0x3fb00000u) return GENERAL;
+  return lo >= 0x26f00000u ? SOFT : FAST;
+}
+// the form all lanes allow
+__device__ __forceinline__ int warp_form(int f) { return (int)__reduce_min_sync(0xffffffffu, (unsigned)f); }
+// a product on the integer pipes (SOFT) or on the unit
+template <int FORM> __device__ __forceinline__ double prod(const Unit &U, double x, double y) {
+  return FORM == SOFT ? mulz(x, y) : U.mul(x, y);
 }
 
 // One interface: speeds, and the waves of the two acoustic families
@@ -152,17 +173,20 @@ __device__ __forceinline__ bool face_general(double beta2, const double L[2 + NT
   return nonreal;
 }
 
-template <int NT>
+template <int FORM, int NT>
 __device__ __forceinline__ void face_fast(const Par &P, const double L[2 + NT],
                                           const double zL[1 + NT], const double R[2 + NT],
                                           const double zR[1 + NT], Face<NT> &F) {
   const Unit &U = P.U;
   const double S1 = U.add(L[0], R[0]);
   const double S2 = U.add(zL[0], zR[0]);
-  const double Phi = U.add(mulz(P.bh, U.add(S1, -2.0)), 1.0);
-  const double rs = int64f::rcp_mid(S1);
-  const double u = mulz(S2, rs);
-  const double D = U.add(U.sub(mulz(u, u), mulz(S2, u)), Phi);
+  const double Phi = U.add(prod<FORM>(U, P.bh, U.add(S1, -2.0)), 1.0);
+  // 1/S1 with the halves moved out (SOFT), or 1/Z1 and the halves taken as defined
+  const double rs = FORM == SOFT ? int64f::rcp_mid(S1) : int64f::twice(int64f::rcp_mid(S1));
+  const double Z2 = FORM == SOFT ? S2 : U.mul(0.5, S2);
+  const double T2 = FORM == SOFT ? S2 : U.add(Z2, Z2);
+  const double u = prod<FORM>(U, Z2, rs);
+  const double D = U.add(U.sub(prod<FORM>(U, u, u), prod<FORM>(U, T2, u)), Phi);
   const double c = int64f::sqrt_mid(D);
   F.s0 = U.add(u, c);
   F.s1 = U.sub(u, c);
@@ -171,18 +195,19 @@ __device__ __forceinline__ void face_fast(const Par &P, const double L[2 + NT],
   const double h = int64f::half_of(rc);
   const double d1 = U.sub(R[0], L[0]);
   const double d2 = U.sub(R[1], L[1]);
-  const double e0 = U.sub(F.s0, S2), e1 = U.sub(S2, F.s1);
-  F.a1 = mulz(U.sub(d2, mulz(F.s1, d1)), h);
-  F.a2 = mulz(U.sub(mulz(F.s0, d1), d2), h);
-  F.w01 = mulz(F.a1, F.s0);
-  F.w11 = mulz(F.a2, F.s1);
+  const double e0 = U.sub(F.s0, T2), e1 = U.sub(T2, F.s1);
+  F.a1 = prod<FORM>(U, U.sub(d2, prod<FORM>(U, F.s1, d1)), h);
+  F.a2 = prod<FORM>(U, U.sub(prod<FORM>(U, F.s0, d1), d2), h);
+  F.w01 = prod<FORM>(U, F.a1, F.s0);
+  F.w11 = prod<FORM>(U, F.a2, F.s1);
 #pragma unroll
   for (int k = 0; k < NT; k++) {
-    const double v = mulz(U.add(zL[1 + k], zR[1 + k]), rs);
-    const double r1 = mulz(mulz(v, e0), rc);
-    const double r2 = mulz(mulz(v, e1), rc);
-    F.w0[k] = mulz(F.a1, r1);
-    F.w1[k] = mulz(F.a2, r2);
+    const double S = U.add(zL[1 + k], zR[1 + k]);
+    const double v = prod<FORM>(U, FORM == SOFT ? S : U.mul(0.5, S), rs);
+    const double r1 = prod<FORM>(U, prod<FORM>(U, v, e0), rc);
+    const double r2 = prod<FORM>(U, prod<FORM>(U, v, e1), rc);
+    F.w0[k] = prod<FORM>(U, F.a1, r1);
+    F.w1[k] = prod<FORM>(U, F.a2, r2);
     F.w2[k] = U.sub(U.sub(U.sub(R[2 + k], L[2 + k]), F.w0[k]), F.w1[k]);
   }
 }
@@ -210,12 +235,16 @@ __device__ __forceinline__ double phi_fast(const Unit &U, double num, double den
   nb = on ? nb : 0x3ff0000000000000ull;
   db = on ? db : 0x3ff0000000000000ull;
   double theta;
-  if (int64f::mid((int64f::u32)(nb >> 32)) && int64f::mid((int64f::u32)(db >> 32)))
-    theta = int64f::div_mid(nb, db);
-  else
+  int64f::u64 b;             // 2 theta
+  const int64f::u32 nh = (int64f::u32)(nb >> 32), dh = (int64f::u32)(db >> 32);
+  if (nh >= 0x00100000u && dh >= 0x00100000u && nh - dh + (900u << 20) < (1800u << 20)) {
+    theta = int64f::div_normal(nb, db);
+    b = int64f::bits_of(int64f::twice(theta));
+  } else {
     theta = int64f::of_bits(nb) / int64f::of_bits(db);
+    b = int64f::bits_of(theta + theta);
+  }
   const int64f::u64 a = int64f::bits_of(int64f::half_of(U.add(theta, 1.0)));
-  const int64f::u64 b = int64f::bits_of(theta) + 0x10000000000000ull;
   int64f::u64 m = a < b ? a : b;
   m = hi_of(theta) >= 0x40080000u ? 0x4000000000000000ull : m;
   m = on ? m : 0;
@@ -262,8 +291,8 @@ __device__ __forceinline__ void flux_general(const Face<NT> &I, const Face<NT> &
   }
 }
 
-// tiny: a limiter value was met with which G may be subnormal
-template <int LIM, int NT>
+// tiny: halves of G may be subnormal
+template <int FORM, int LIM, int NT>
 __device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const Face<NT> &Lf,
                                           const Face<NT> &Rf, Flux<NT> &o, bool &tiny) {
   const Unit &U = P.U;
@@ -272,10 +301,10 @@ __device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const
   o.ap[0] = I.w01;
   o.am[1] = U.mul(I.s1, I.w11);
   o.ap[1] = U.mul(I.s0, I.w01);
-  double d0 = U.add(mulz(I.a1, I.a1), mulz(I.w01, I.w01));
-  double n0 = U.add(mulz(Lf.a1, I.a1), mulz(Lf.w01, I.w01));
-  double d1 = U.add(mulz(I.a2, I.a2), mulz(I.w11, I.w11));
-  double n1 = U.add(mulz(Rf.a2, I.a2), mulz(Rf.w11, I.w11));
+  double d0 = U.add(prod<FORM>(U, I.a1, I.a1), prod<FORM>(U, I.w01, I.w01));
+  double n0 = U.add(prod<FORM>(U, Lf.a1, I.a1), prod<FORM>(U, Lf.w01, I.w01));
+  double d1 = U.add(prod<FORM>(U, I.a2, I.a2), prod<FORM>(U, I.w11, I.w11));
+  double n1 = U.add(prod<FORM>(U, Rf.a2, I.a2), prod<FORM>(U, Rf.w11, I.w11));
 #pragma unroll
   for (int k = 0; k < NT; k++) {
     // the transverse wave joins the fluctuation of the side it moves to
@@ -283,10 +312,10 @@ __device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const
     const double t = U.add(neg ? X : Y, U.mul(I.u, I.w2[k]));
     o.am[2 + k] = neg ? t : X;
     o.ap[2 + k] = neg ? Y : t;
-    d0 = U.add(d0, mulz(I.w0[k], I.w0[k]));
-    n0 = U.add(n0, mulz(Lf.w0[k], I.w0[k]));
-    d1 = U.add(d1, mulz(I.w1[k], I.w1[k]));
-    n1 = U.add(n1, mulz(Rf.w1[k], I.w1[k]));
+    d0 = U.add(d0, prod<FORM>(U, I.w0[k], I.w0[k]));
+    n0 = U.add(n0, prod<FORM>(U, Lf.w0[k], I.w0[k]));
+    d1 = U.add(d1, prod<FORM>(U, I.w1[k], I.w1[k]));
+    n1 = U.add(n1, prod<FORM>(U, Rf.w1[k], I.w1[k]));
   }
   const double as1 = -I.s1, asu = fabs(I.u);
   const double c0 = U.mul(U.mul(I.s0, U.sub(1.0, U.mul(P.lam, I.s0))), phi_fast<LIM>(U, n0, d0, tiny));
@@ -298,8 +327,10 @@ __device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const
   for (int k = 0; k < NT; k++) {
     const double w = neg ? Rf.w2[k] : Lf.w2[k];
     const double c2 =
-        U.mul(fu, phi_fast<LIM>(U, mulz(w, I.w2[k]), mulz(I.w2[k], I.w2[k]), tiny));
+        U.mul(fu, phi_fast<LIM>(U, U.mul(w, I.w2[k]), U.mul(I.w2[k], I.w2[k]), tiny));
     o.G[2 + k] = U.add(U.add(U.mul(c0, I.w0[k]), U.mul(c1, I.w1[k])), U.mul(c2, I.w2[k]));
+    if (FORM == SOFT)
+      tiny |= (int64f::bits_of(o.G[2 + k]) & 0x7fffffffffffffffull) - 1 < (123ull << 52);
   }
 }
 
@@ -345,7 +376,7 @@ __device__ __forceinline__ void speed_max(unsigned long long &m, const Face<NT> 
 __device__ __forceinline__ double up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ double down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
-template <int LIM, int NT, int CPL, bool FAST>
+template <int FORM, int LIM, int NT, int CPL>
 __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2 + NT], int g, int n,
                                              unsigned long long &smax, bool &nonreal,
                                              double o[CPL][2 + NT], int flo, int fhi) {
@@ -353,7 +384,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
   double z[CPL][1 + NT], ql[2 + NT], zl[1 + NT];
 #pragma unroll
   for (int i = 0; i < CPL; i++) {
-    if (FAST) z_fast<NT>(P, q[i], z[i]);
+    if (FORM) z_fast<NT>(P, q[i], z[i]);
     else z_general<NT>(q[i], z[i]);
   }
 #pragma unroll
@@ -365,11 +396,11 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
   for (int i = 0; i < CPL; i++) {
     const double *L = i ? q[i ? i - 1 : 0] : ql, *zL = i ? z[i ? i - 1 : 0] : zl;
     bool nr = false;
-    if (FAST) face_fast<NT>(P, L, zL, q[i], z[i], F[i]);
+    if (FORM) face_fast<FORM, NT>(P, L, zL, q[i], z[i], F[i]);
     else nr = face_general<NT>(P.beta2, L, zL, q[i], z[i], F[i]);
     const int gl = g + i - 1;                      // left cell of the face
     if (i > 0 || lane > 0) {
-      if (!FAST && gl >= -2 && gl <= n) nonreal |= nr;
+      if (!FORM && gl >= -2 && gl <= n) nonreal |= nr;
       if (gl >= -1 && gl <= n - 1) speed_max(smax, F[i]);
     }
   }
@@ -377,7 +408,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
   Face<NT> A, B;
   A.a1 = up1(F[CPL - 1].a1); A.w01 = up1(F[CPL - 1].w01);
   B.a2 = down1(F[0].a2); B.w11 = down1(F[0].w11);
-  if (!FAST) {
+  if (!FORM) {
     A.a2 = up1(F[CPL - 1].a2); A.w11 = up1(F[CPL - 1].w11);
     B.a1 = down1(F[0].a1); B.w01 = down1(F[0].w01);
   }
@@ -385,7 +416,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
   for (int k = 0; k < NT; k++) {
     A.w0[k] = up1(F[CPL - 1].w0[k]); A.w2[k] = up1(F[CPL - 1].w2[k]);
     B.w1[k] = down1(F[0].w1[k]); B.w2[k] = down1(F[0].w2[k]);
-    if (!FAST) {
+    if (!FORM) {
       A.w1[k] = up1(F[CPL - 1].w1[k]);
       B.w0[k] = down1(F[0].w0[k]);
     }
@@ -395,14 +426,14 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
 #pragma unroll
   for (int i = 0; i < CPL; i++) {
     const Face<NT> &Lf = i ? F[i ? i - 1 : 0] : A, &Rf = i + 1 < CPL ? F[i + 1 < CPL ? i + 1 : 0] : B;
-    if (FAST) flux_fast<LIM, NT>(P, F[i], Lf, Rf, X[i], tiny);
+    if (FORM) flux_fast<FORM, LIM, NT>(P, F[i], Lf, Rf, X[i], tiny);
     else flux_general<LIM, NT>(F[i], Lf, Rf, P.lam, X[i]);
     if (g + i >= flo && g + i <= fhi) {
 #pragma unroll
       for (int k = 0; k < 2 + NT; k++) X[i].G[k] = 0.0;
     }
   }
-  const bool half = FAST && !__any_sync(0xffffffffu, tiny);
+  const bool half = FORM == SOFT && !__any_sync(0xffffffffu, tiny);
   double am[2 + NT], G[2 + NT];                    // the next lane's first face
 #pragma unroll
   for (int k = 0; k < 2 + NT; k++) {
@@ -423,11 +454,13 @@ template <int LIM, int NT, int CPL>
 __device__ __forceinline__ void lanes_step(const Par &P, const double q[CPL][2 + NT], int g, int n,
                                            unsigned long long &smax, bool &nonreal,
                                            double o[CPL][2 + NT], int flo = 1, int fhi = 0) {
-  bool t = P.ok;
+  int f = P.ok ? SOFT : GENERAL;
 #pragma unroll
-  for (int i = 0; i < CPL; i++) t = t && tame_cell<NT>(q[i]);
-  if (__all_sync(0xffffffffu, t)) lanes_update<LIM, NT, CPL, true>(P, q, g, n, smax, nonreal, o, flo, fhi);
-  else lanes_update<LIM, NT, CPL, false>(P, q, g, n, smax, nonreal, o, flo, fhi);
+  for (int i = 0; i < CPL; i++) f = min(f, form_of<NT>(q[i]));
+  f = warp_form(f);
+  if (f == SOFT) lanes_update<SOFT, LIM, NT, CPL>(P, q, g, n, smax, nonreal, o, flo, fhi);
+  else if (f == FAST) lanes_update<FAST, LIM, NT, CPL>(P, q, g, n, smax, nonreal, o, flo, fhi);
+  else lanes_update<GENERAL, LIM, NT, CPL>(P, q, g, n, smax, nonreal, o, flo, fhi);
 }
 
 // ---------------------------------------------------------------------------
@@ -439,13 +472,13 @@ template <int LIM, int NT> struct March {
   double c1[2 + NT], c2[2 + NT], z1[1 + NT];
   Face<NT> f1, f2;            // faces j - 1 and j - 2
   double ap[2 + NT], G[2 + NT];
-  int run;                    // tame cells in a row, the same in all lanes
+  int fast, soft;             // cells in a row that allow these forms, the same in all lanes
   bool lhalf;                 // the left face's G may be halved after the fact
   unsigned long long smax;
   bool nonreal;
 
   __device__ __forceinline__ void init() {
-    run = 0;
+    fast = soft = 0;
     lhalf = true;
     smax = 0;
     nonreal = false;
@@ -455,33 +488,36 @@ template <int LIM, int NT> struct March {
   __device__ __forceinline__ bool push(const Par &P, int j, const double q[2 + NT],
                                        double out[2 + NT], bool count_speed, bool count_real,
                                        bool plain) {
-    run = __all_sync(0xffffffffu, P.ok && tame_cell<NT>(q)) ? run + 1 : 0;
-    // this cell and the four before it
-    if (run > (j < 4 ? j : 4)) step<true>(P, j, q, out, count_speed, count_real, plain);
-    else step<false>(P, j, q, out, count_speed, count_real, plain);
+    const int f = warp_form(P.ok ? form_of<NT>(q) : GENERAL);
+    fast = f >= FAST ? fast + 1 : 0;
+    soft = f == SOFT ? soft + 1 : 0;
+    const int need = j < 4 ? j : 4;                // this cell and the four before it
+    if (soft > need) step<SOFT>(P, j, q, out, count_speed, count_real, plain);
+    else if (fast > need) step<FAST>(P, j, q, out, count_speed, count_real, plain);
+    else step<GENERAL>(P, j, q, out, count_speed, count_real, plain);
     return j >= 4;
   }
-  template <bool FAST>
+  template <int FORM>
   __device__ __forceinline__ void step(const Par &P, int j, const double q[2 + NT],
                                        double out[2 + NT], bool count_speed, bool count_real,
                                        bool plain) {
     double z[1 + NT];
-    if (FAST) z_fast<NT>(P, q, z);
+    if (FORM) z_fast<NT>(P, q, z);
     else z_general<NT>(q, z);
     if (j > 0) {
       Face<NT> f;
-      if (FAST) face_fast<NT>(P, c1, z1, q, z, f);
+      if (FORM) face_fast<FORM, NT>(P, c1, z1, q, z, f);
       else {
         const bool nr = face_general<NT>(P.beta2, c1, z1, q, z, f);
         if (count_real) nonreal |= nr;
       }
       if (j >= 3) {
         Flux<NT> X;
-        bool half = FAST;
-        if (FAST) {
+        bool half = FORM == SOFT;
+        if (FORM) {
           bool tiny = false;
-          flux_fast<LIM, NT>(P, f1, f2, f, X, tiny);
-          half = !__any_sync(0xffffffffu, tiny);
+          flux_fast<FORM, LIM, NT>(P, f1, f2, f, X, tiny);
+          half = half && !__any_sync(0xffffffffu, tiny);
         } else {
           flux_general<LIM, NT>(f1, f2, f, P.lam, X);
         }

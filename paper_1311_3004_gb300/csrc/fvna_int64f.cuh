@@ -131,9 +131,9 @@ INT64F_FN double rcp_mid(double a) {
   return of_bits(Q + ((u64)e << 32));
 }
 
-// n/d for mid(n), mid(d) and |d| < 2^510 (so that the quotient is normal).
-// The approximation is (-4.1, 4.1) units off after the normalising shift.
-INT64F_FN double div_mid(u64 nb, u64 db) {
+// n/d for normal n and d whose exponents differ by less than 1000 (so that the
+// quotient is normal).  The approximation is (-4.1, 4.1) units off after the normalising shift.
+INT64F_FN double div_normal(u64 nb, u64 db) {
   const u64 M = significand(db), N = significand(nb);
   const u64 q = mul_hi(N << 11, recip63(M << 11));  // 62 fractional bits, in (1/2, 2)
   const u32 lt = 1u - (u32)(q >> 62);               // 1: the quotient is below 1

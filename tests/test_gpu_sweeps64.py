@@ -43,6 +43,16 @@ def _states():
     q[1:] = rng.choice([-1, 1], size=q[1:].shape) * 2.0 ** rng.uniform(-1074, -5, size=q[1:].shape)
     q[1:][rng.random(q[1:].shape) < 0.2] = 0.0
     out["scattered"] = q
+    # each of the fast form's ranges by itself: down to 2^-400, and from there to the subnormals
+    for name, lo, hi in (("small", -399, -5), ("smaller", -1070, -402)):
+        q = smooth.copy()
+        q[1:] = rng.choice([-1, 1], size=q[1:].shape) * 2.0 ** rng.uniform(lo, hi,
+                                                                           size=q[1:].shape)
+        q[1:][rng.random(q[1:].shape) < 0.1] = 0.0
+        out[name] = q
+        q = q.copy()
+        q[0] = 1.0
+        out[name + " at rest"] = q
     # a pulse at rest: exact zeros around it, then a numerical precursor that decays without end
     q = wl.centred_gaussian(n, m, 1e-3, 2.0)
     out["precursor"] = q
