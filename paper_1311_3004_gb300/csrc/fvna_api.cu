@@ -339,6 +339,12 @@ static double tile_cost(long long tiles, int sms, int per_tile, int want) {
   return per_sm * per_tile / fill;
 }
 static int pick_tile_x32(int n, const fvna_domain *d, int sms) {
+  // below two million cells the segments with the lanes along x1, which leave
+  // no lane a line to march (1024^2 cells 16.5 us against 17.4 to 22 for the
+  // marched tiles, 257 x 129 9.3 against 10.3; at 2048^2 38.5 against 34.4)
+  long long cells = 0;
+  for (int k = 0; k < n; k++) cells += (long long)d[k].nx * d[k].ny;
+  if (cells < 2000000) return X32H_TILE;
   int best = 64;
   double best_cost = 1e300;
   for (int tx : {64, 32, 16}) {
@@ -351,14 +357,25 @@ static int pick_tile_x32(int n, const fvna_domain *d, int sms) {
   }
   return best;
 }
-// x2 sweep: each warp marches its columns row after row, so the sweep runs
-// at the pace of its warps' latency and of its slowest tiles (those at a
-// border take the general path); a height whose marched rows (ty + 6) fill
-// whole 8-row chunks.  The smallest, 10 (two chunks, both loaded when the
-// tile starts, and the most tiles to balance the warps with), measured
-// fastest on the 2048^2 pulse (53.6 us against 56.2 for 18 and 68.7 for 22;
-// taller tiles and mixed heights were slower still).
-static int pick_tile_y32() { return 10; }
+// x2 sweep: a tile of ty rows marches ty + 6, so the work falls with the
+// height as (ty + 6)/ty while the last tiles, which nothing overlaps, take
+// ty + 6 steps.  Measured, the sweep takes about 5.5 us per million marched
+// cells and 0.9 us per step of its last tiles; heights whose marched rows fill
+// whole 8-row chunks.  (us for ty = 10, 18, 26, 34, 42: 2048^2 49.7, 53, 62,
+// 74, 82; 3000^2 90, 82, 80, 93, 102; 4096^2 154, 136, 130, 130, 130; 39
+// million cells in 48 domains 385, 341, 324, 320, 320.  257 x 129: 25
+// at 10 and 16 at 2.)
+static int pick_tile_y32(int n, const fvna_domain *d) {
+  double cells = 0.0;
+  for (int k = 0; k < n; k++) cells += 1e-6 * d[k].nx * (double)d[k].ny;
+  int best = 10;
+  double best_cost = 1e300;
+  for (int ty : {2, 10, 18, 26, 34, 42}) {
+    const double c = 5.5 * cells * (ty + 6) / ty + 0.9 * (ty + 6);
+    if (c < best_cost) { best_cost = c; best = ty; }
+  }
+  return best;
+}
 
 static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
                      const double *const *q0, int q0_on_device, void *stream, fvna_ctx *c) {
@@ -381,7 +398,7 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
     c->tile_y = t64.tile_y;
   } else {
     c->tile_x = cfg->tile_x ? cfg->tile_x : pick_tile_x32(n, doms, sms);
-    c->tile_y = cfg->tile_y ? cfg->tile_y : pick_tile_y32();
+    c->tile_y = cfg->tile_y ? cfg->tile_y : pick_tile_y32(n, doms);
   }
   // border values evaluated once per step: binary64 domains driven on the
   // x1-low border (HIFU) keep a drive buffer; binary32 domains with any

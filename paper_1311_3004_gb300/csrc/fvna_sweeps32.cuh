@@ -679,7 +679,7 @@ __device__ __forceinline__ int y32_tile(const StepArgs &A, const DomDev &D, DomS
   const int klo = HALO_Y, khi = min(TY + HALO_Y, D.ny - y0 + HALO_Y);
   const int nlo = max(1, 2 - y0), nhi = D.ny + 4 - y0;
   int glo = 1, ghi = 0;
-  if (axi && D.y0 == 0.0 && y0 == 0) { glo = HALO_Y; ghi = HALO_Y + AXIS_FACES - 1; }
+  if (axi && D.y0 == 0.0) { glo = HALO_Y - y0; ghi = glo + AXIS_FACES - 1; }
   March<LIM, COMP, SPEC> m;
   m.init((float)A.beta, S->lam32);
   YSrc src;
