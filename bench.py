@@ -227,7 +227,8 @@ _SWEEP_SOURCES = ["fvna_api.cu", "fvna_device.cuh", "fvna_face64.cuh", "fvna_fp3
                   "fvna_sweeps32.cuh", "fvna_types.h", "fvna_x2.cuh"]
 
 
-_SWEEP3_SOURCES = ["fvna_3d.cuh", "fvna_3d.inc", "fvna_3d_sweep64.cuh", "fvna_3d32.cu", "fvna_3d64.cu", "fvna_api3d.cu",
+_SWEEP3_SOURCES = ["fvna_3d.cuh", "fvna_3d.inc", "fvna_3d_sweep32.cuh", "fvna_3d_sweep64.cuh",
+                   "fvna_3d32.cu", "fvna_3d64.cu", "fvna_api3d.cu", "fvna_x2.cuh",
                    "fvna_face64.cuh", "fvna_int64f.cuh", "fvna_launch3.h"]
 
 
@@ -264,7 +265,7 @@ _TRAFFIC_KEYS = [
 ]
 # the 3D kernels (k3_sweep_v serves the x2 and the x3 sweep: one figure for both)
 _TRAFFIC_KEYS3 = [
-    (r"k3_sweep_x<float", "k3_sweep_x_fp32"), (r"k3_sweep_v<float", "k3_sweep_v_fp32"),
+    (r"k3_sweep_xp<", "k3_sweep_x_fp32"), (r"k3_sweep_vp<", "k3_sweep_v_fp32"),
     (r"k3_source<float", "k3_source_fp32"), (r"k3_sweep64<", "k3_sweep_x_fp64"),
     (r"k3_source<double", "k3_source_fp64"),
 ]

@@ -357,7 +357,8 @@ typedef struct fvna3_ctx fvna3_ctx;
  *         nu_w, nu_max, dt_fixed, steps_per_graph and compensated as in 2D;
  *         geometry must be FVNA_CARTESIAN and splitting FVNA_SPLIT_GODUNOV;
  *         sweeps is not read (dom->substeps selects sub-steps); tile_y is
- *         the height of the binary32 x2/x3 sweeps' tiles (0: 64)
+ *         the height of the binary32 x2/x3 sweeps' tiles (0: picked
+ *         from the domain's size)
  *   dom   the domain (borrowed, copied)
  *   q0    4*nx*ny*nz binary64 total variables in the layout above (borrowed,
  *         copied; device memory if q0_on_device)

@@ -34,7 +34,8 @@ struct fvna3_ctx {
   cudaGraphExec_t gexec = nullptr;
   int gsteps = 32;
   int prec = 0;
-  int blocks_x = 1, blocks_v = 1, blocks_e = 1;
+  int blocks_x = 1, blocks_v[3] = {1, 1, 1}, blocks_e = 1;
+  int tile[3] = {0, 64, 64};   // heights of the binary32 x2 and x3 sweeps' tiles
   int kernels_per_step = 0;
   long long launches = 0;
 };
@@ -88,8 +89,9 @@ int enqueue_step(fvna3_ctx *c, cudaStream_t s, cudaEvent_t *ev) {
   for (int d = 0; d < 3; d++) {
     if (sw & (1 << d)) {
       Args3 a = with_planes(c, cur, nxt, d);
+      a.tile = c->tile[d];
       if (fp64(c)) CK3(launch3_sweep_64(a, c->blocks_x, s));
-      else CK3(d == 0 ? launch3_sweep_x_32(a, c->blocks_x, s) : launch3_sweep_v_32(a, c->blocks_v, s));
+      else CK3(d == 0 ? launch3_sweep_x_32(a, c->blocks_x, s) : launch3_sweep_v_32(a, c->blocks_v[d], s));
       std::swap(cur, nxt);
     }
     CK3(mark(1 + d));
@@ -198,6 +200,23 @@ int validate3(const fvna_config *c, const fvna_domain3 *d, const double *q0) {
   return FVNA_OK;
 }
 
+// Height of the binary32 x2 or x3 sweep's tiles: a warp marches tile + 4 cells
+// a tile, and the sweep lasts as many rounds as the tiles make over the
+// resident warps (256^3: heights 64 take 3 rounds of 68, 37 four of 41).
+int pick_tile3(const Dom3 &D, int dir, int warps) {
+  const int n = dir == 1 ? D.ny : D.nz;
+  int best = 4;
+  long long best_cost = -1;
+  for (int t = std::min(n, 4); t <= std::min(n, 160); t++) {
+    const long long cost = (items3_32(D, dir, t) + warps - 1) / warps * (t + 4);
+    if (best_cost < 0 || cost < best_cost) {
+      best = t;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 int init3(const fvna_config *cfg, const fvna_domain3 *dom, const double *q0, int q0_on_device,
           void *stream, fvna3_ctx *c) {
   c->cfg = *cfg;
@@ -236,23 +255,22 @@ int init3(const fvna_config *cfg, const fvna_domain3 *dom, const double *q0, int
   a.nu_w = cfg->nu_w; a.nu_max = cfg->nu_max; a.dt_fixed = cfg->dt_fixed;
   a.limiter = cfg->limiter;
   a.comp = !fp64(c) && cfg->compensated ? 1 : 0;
-  a.tile = cfg->tile_y ? cfg->tile_y : 64;
 
   // persistent grids: the sweeps' tiles handed out grid-stride
   int dev = 0, sms = 0, ox = 0, ov = 0;
   CK3(cudaGetDevice(&dev));
   CK3(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  if (!fp64(c)) occupancy3_32(cfg->limiter, a.comp, &ox, &ov);
-  const int tx = tile_x3_32();
-  const long long xt = (long long)((D.nx + tx - 1) / tx) * D.ny * (long long)D.nz;
-  const long long vt2 = (long long)((D.nx + 31) / 32) * ((D.ny + a.tile - 1) / a.tile) * D.nz;
-  const long long vt3 = (long long)((D.nx + 31) / 32) * ((D.nz + a.tile - 1) / a.tile) * D.ny;
-  const long long vt = std::max(vt2, vt3);
-  c->blocks_x = (int)std::max<long long>(1, std::min<long long>((xt + 3) / 4,
-                                                                (long long)std::max(ox, 1) * sms));
-  c->blocks_v = (int)std::max<long long>(1, std::min<long long>((vt + 3) / 4,
-                                                                (long long)std::max(ov, 1) * sms));
-  if (fp64(c)) c->blocks_x = occupancy3_64(cfg->limiter) * sms;
+  if (fp64(c)) {
+    c->blocks_x = occupancy3_64(cfg->limiter) * sms;
+  } else {
+    occupancy3_32(cfg->limiter, a.comp, &ox, &ov);
+    const int most_x = std::max(ox, 1) * sms, most_v = std::max(ov, 1) * sms;
+    c->blocks_x = (int)std::min<long long>((items3_32(D, 0, 0) + 3) / 4, most_x);
+    for (int d = 1; d < 3; d++) {
+      c->tile[d] = cfg->tile_y ? cfg->tile_y : pick_tile3(D, d, 4 * most_v);
+      c->blocks_v[d] = (int)std::min<long long>((items3_32(D, d, c->tile[d]) + 3) / 4, most_v);
+    }
+  }
   c->blocks_e = std::max(1, std::min((int)((D.plane + 255) / 256), 16 * sms));
   c->kernels_per_step = kernels_per_step(substeps(c));
 

@@ -8,7 +8,7 @@
 namespace fvna {
 namespace d3 {
 
-int tile_x3_32();
+long long items3_32(const Dom3 &D, int dir, int tile);
 // binary64: one sweep kernel (Args3::dir says which); resident blocks per SM,
 // and a launch of at most `blocks` blocks
 int occupancy3_64(int lim);
