@@ -239,23 +239,31 @@ constexpr int X3_OUT = 60;
 // Source: forward Euler with the 7-point Laplacian of z = (q2, q3, q4)/q1,
 // summed as ((W + E) + (S + N) - 4 C) + ((B + T) - 2 C).
 // ---------------------------------------------------------------------------
-// state of cell (i, j, k), ghost cells by the border rules (the normal
-// momentum of a mirrored cell negated), and its velocity z = (q2, q3, q4)/q1
+// One column (i, j) along x3, its ghost columns by the border rules: the
+// mapped offset in a plane and which momenta a mirrored cell negates.
+struct Column3 {
+  long long off;
+  bool fx, fy;
+  __device__ __forceinline__ Column3(const Dom3 &D, int i, int j) {
+    const int ci = map_cell(i, D.nx, D.bc[0], D.bc[1], fx);
+    const int cj = map_cell(j, D.ny, D.bc[2], D.bc[3], fy);
+    off = (long long)cj * D.pitch + ci;
+  }
+};
+// state of a column's cell at plane k
 template <class T>
-__device__ __forceinline__ void qat(const Args3 &A, int i, int j, int k, T q[4]) {
-  const Dom3 &D = A.d;
-  bool fx = false, fy = false, fz = false;
-  int ci = map_cell(i, D.nx, D.bc[0], D.bc[1], fx);
-  int cj = map_cell(j, D.ny, D.bc[2], D.bc[3], fy);
-  int ck = map_cell(k, D.nz, D.bc[4], D.bc[5], fz);
-  long long off = ((long long)ck * D.ny + cj) * D.pitch + ci;
-  const T *const *in = (const T *const *)A.in;
+__device__ __forceinline__ void qat(const Dom3 &D, const T *const in[4], const Column3 &c, int k,
+                                    T q[4]) {
+  bool fz = false;
+  if (k < 0 || k >= D.nz) k = map_cell(k, D.nz, D.bc[4], D.bc[5], fz);
+  const long long off = (long long)k * D.ny * D.pitch + c.off;
 #pragma unroll
   for (int f = 0; f < 4; f++) q[f] = in[f][off];
-  if (fx) q[1] = -q[1];
-  if (fy) q[2] = -q[2];
+  if (c.fx) q[1] = -q[1];
+  if (c.fy) q[2] = -q[2];
   if (fz) q[3] = -q[3];
 }
+// its velocity z = (q2, q3, q4)/q1
 template <class T> __device__ __forceinline__ void zof3(const T q[4], T z[3]) {
   T r = inv_q1(q[0]);
   z[0] = q[1] * r;
@@ -281,7 +289,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
   __shared__ T sz[3][SRC3_TY + 2][SRC3_TX + 2];
   const int tx = threadIdx.x % SRC3_TX, ty = threadIdx.x / SRC3_TX;
   const T coef = sizeof(T) == 8 ? (T)S->coef : (T)S->coef32;
-  T *const *out = (T *const *)A.out;
+  const T *const in[4] = {(const T *)A.in[0], (const T *)A.in[1], (const T *)A.in[2],
+                          (const T *)A.in[3]};
+  T *const out[4] = {(T *)A.out[0], (T *)A.out[1], (T *)A.out[2], (T *)A.out[3]};
   // the ring cell this thread forms (threads 0 .. 2 (TX + TY) - 1): the
   // x1-low and x1-high columns, then the x2-low and x2-high rows
   const int h = threadIdx.x;
@@ -295,19 +305,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
   for (int jt = blockIdx.y; jt < ntj; jt += gridDim.y) {
     const int j0 = jt * SRC3_TY, j = j0 + ty;
     const bool own = i < D.nx && j < D.ny;
-    const int hi = i0 - 1 + hx, hj = j0 - 1 + hy;
+    const Column3 col(D, i, j), ring(D, i0 - 1 + hx, j0 - 1 + hy);
     for (int kc = blockIdx.z; kc < nkc; kc += gridDim.z) {
       const int k0 = kc * SRC3_KCH, k1 = min(D.nz, k0 + SRC3_KCH);
       T zb[3], zc[3], zt[3], qc[4], qt[4], hq[4];
-      qat<T>(A, i, j, k0 - 1, qc);
+      qat<T>(D, in, col, k0 - 1, qc);
       zof3<T>(qc, zb);
-      qat<T>(A, i, j, k0, qc);
+      qat<T>(D, in, col, k0, qc);
       zof3<T>(qc, zc);
-      qat<T>(A, i, j, k0 + 1, qt);
-      if (hx >= 0) qat<T>(A, hi, hj, k0, hq);
+      qat<T>(D, in, col, k0 + 1, qt);
+      if (hx >= 0) qat<T>(D, in, ring, k0, hq);
       for (int k = k0; k < k1; k++) {
         T qn[4];
-        if (k + 1 < k1) qat<T>(A, i, j, k + 2, qn);
+        if (k + 1 < k1) qat<T>(D, in, col, k + 2, qn);
         zof3<T>(qt, zt);
 #pragma unroll
         for (int f = 0; f < 3; f++) sz[f][ty + 1][tx + 1] = zc[f];
@@ -316,7 +326,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
           zof3<T>(hq, zh);
 #pragma unroll
           for (int f = 0; f < 3; f++) sz[f][hy][hx] = zh[f];
-          if (k + 1 < k1) qat<T>(A, hi, hj, k + 1, hq);
+          if (k + 1 < k1) qat<T>(D, in, ring, k + 1, hq);
         }
         __syncthreads();
         if (own) {
