@@ -60,6 +60,7 @@ struct Args3 {
   void *out[4];           // planes written by the launch
   double beta, delta, dx, nu_w, nu_max, dt_fixed;
   int limiter, comp, dir, tile;   // dir: 0 x1, 1 x2, 2 x3; tile: TY of the x2/x3 sweeps
+  int chunk;                      // planes a block of the source marches
 };
 
 // ---------------------------------------------------------------------------
@@ -272,7 +273,12 @@ template <class T> __device__ __forceinline__ void zof3(const T q[4], T z[3]) {
 }
 
 // One block marches a tile of SRC3_TX x SRC3_TY cells of the (x1, x2) plane
-// along x3 through a chunk of SRC3_KCH planes.  Every cell's velocity z is
+// along x3 through a chunk of planes.  The velocities of a plane alternate
+// between two buffers, so that one barrier a plane is enough; six blocks an SM
+// hide the loads' latency (256^3 binary32: 152 us, four blocks 176, with two
+// barriers 174; 79 at the copy rate).  A chunk costs two planes of start-up and
+// is a block's serial length: 16 planes, fewer where the domain has too few
+// blocks (64^3: 20.5 us in chunks of 16, 10.2 in chunks of 2).  Every cell's velocity z is
 // formed once per plane: the tile's cells and a one-cell ring around it go
 // to shared memory for the x1 and x2 neighbours (the ring's cells are the
 // border rules' ghosts where the tile meets a border), and each thread keeps
@@ -280,13 +286,14 @@ template <class T> __device__ __forceinline__ void zof3(const T q[4], T z[3]) {
 // thread needs next (its own cell two planes ahead, its ring cell one plane
 // ahead) is loaded while the current plane is formed.  Threads of a tile
 // that overhangs the domain form ghost or clamped cells and store nothing.
-constexpr int SRC3_TX = 32, SRC3_TY = 8, SRC3_KCH = 16;
+constexpr int SRC3_TX = 32, SRC3_TY = 8;
+constexpr int SRC3_BLOCKS = 608;   // blocks wanted before chunks are shortened: four an SM
 template <class T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 2) k3_source(Args3 A) {
   Scal3 *S = A.S;
   if (S->done) return;
   const Dom3 &D = A.d;
-  __shared__ T sz[3][SRC3_TY + 2][SRC3_TX + 2];
+  __shared__ T szs[2][3][SRC3_TY + 2][SRC3_TX + 2];
   const int tx = threadIdx.x % SRC3_TX, ty = threadIdx.x / SRC3_TX;
   const T coef = sizeof(T) == 8 ? (T)S->coef : (T)S->coef32;
   const T *const in[4] = {(const T *)A.in[0], (const T *)A.in[1], (const T *)A.in[2],
@@ -300,14 +307,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
   else if (h < 2 * SRC3_TY) { hx = SRC3_TX + 1; hy = 1 + h - SRC3_TY; }
   else if (h < 2 * SRC3_TY + SRC3_TX) { hx = 1 + h - 2 * SRC3_TY; hy = 0; }
   else if (h < 2 * SRC3_TY + 2 * SRC3_TX) { hx = 1 + h - 2 * SRC3_TY - SRC3_TX; hy = SRC3_TY + 1; }
-  const int ntj = (D.ny + SRC3_TY - 1) / SRC3_TY, nkc = (D.nz + SRC3_KCH - 1) / SRC3_KCH;
+  const int ntj = (D.ny + SRC3_TY - 1) / SRC3_TY, nkc = (D.nz + A.chunk - 1) / A.chunk;
   const int i0 = blockIdx.x * SRC3_TX, i = i0 + tx;
   for (int jt = blockIdx.y; jt < ntj; jt += gridDim.y) {
     const int j0 = jt * SRC3_TY, j = j0 + ty;
     const bool own = i < D.nx && j < D.ny;
     const Column3 col(D, i, j), ring(D, i0 - 1 + hx, j0 - 1 + hy);
     for (int kc = blockIdx.z; kc < nkc; kc += gridDim.z) {
-      const int k0 = kc * SRC3_KCH, k1 = min(D.nz, k0 + SRC3_KCH);
+      const int k0 = kc * A.chunk, k1 = min(D.nz, k0 + A.chunk);
+      __syncthreads();
       T zb[3], zc[3], zt[3], qc[4], qt[4], hq[4];
       qat<T>(D, in, col, k0 - 1, qc);
       zof3<T>(qc, zb);
@@ -316,6 +324,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
       qat<T>(D, in, col, k0 + 1, qt);
       if (hx >= 0) qat<T>(D, in, ring, k0, hq);
       for (int k = k0; k < k1; k++) {
+        T(*const sz)[SRC3_TY + 2][SRC3_TX + 2] = szs[k & 1];
         T qn[4];
         if (k + 1 < k1) qat<T>(D, in, col, k + 2, qn);
         zof3<T>(qt, zt);
@@ -341,7 +350,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k3_source(Args3 A
             out[1 + f][off] = qc[1 + f] + coef * L;
           }
         }
-        __syncthreads();
 #pragma unroll
         for (int f = 0; f < 3; f++) {
           zb[f] = zc[f];
