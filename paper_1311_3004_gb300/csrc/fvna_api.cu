@@ -635,6 +635,7 @@ int fvna_run(fvna_ctx *c, double t_end, long long max_steps, fvna_stats *stats) 
   c->launches += 1;
   long long left = max_steps > 0 ? (max_steps + c->gsteps - 1) / c->gsteps : 0;
   long long batch = 1;
+  bool fresh = false;   // h_scal was read after the last launch
   while (left > 0) {
     long long nb = std::min(batch, left);
     rc = launch_graphs(c, nb);
@@ -642,12 +643,13 @@ int fvna_run(fvna_ctx *c, double t_end, long long max_steps, fvna_stats *stats) 
     left -= nb;
     rc = read_scal(c);
     if (rc != FVNA_OK) return rc;
+    fresh = true;
     bool all_done = true;
     for (int d = 0; d < c->ndom; d++) all_done &= c->h_scal[d].done != 0;
     if (all_done) break;
     batch = std::min<long long>(batch * 2, 64);
   }
-  rc = read_scal(c);
+  if (!fresh) rc = read_scal(c);
   if (rc != FVNA_OK) return rc;
   if (stats) fill_stats(c->h_scal[0], stats);
   return first_status(c);
