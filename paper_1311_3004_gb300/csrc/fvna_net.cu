@@ -209,6 +209,286 @@ __global__ void __launch_bounds__(256) k_net_conv(NetConvArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// The three layers in one kernel, for a forward whose output does not overlap
+// its input.  Persistent blocks keep all weights in shared memory and take
+// tiles of 8 x 32 pixels: the input with a ring of three pixels, the first
+// activation with a ring of two and the second with a ring of one are made in
+// shared memory, so neither activation is read back (both are still written,
+// for a backward).  The rings cost a third more tensor instructions (2,088 of
+// m16n8k16 a tile against 1,568).  Shared memory bounds it (70 % of its
+// cycles, the tensor pipe 48 %), so a warp holds three 16-pixel m-tiles of the
+// hidden layer for each weight fragment, keeps the first and the last layer's
+// weights in registers and shares the last layer's pixels between two rows.
+// Every sum runs over k in the order of k_net_conv: the bits are the same.  One
+// 2048 x 512 field: 157 us in three kernels (39 + 77 + 41), 127 us in this one.
+// ---------------------------------------------------------------------------
+constexpr int F1H = NET_TH + 4, F1W = NET_TW + 4, F1P = F1H * F1W;   // first activation
+constexpr int F2H = NET_TH + 2, F2W = NET_TW + 2, F2P = F2H * F2W;   // second activation
+constexpr int FXH = NET_TH + 6, FXW = NET_TW + 6;                    // input
+constexpr int F1M = F1P / 16, F2M = (F2P + 15) / 16;
+static_assert(F1P % 16 == 0 && F2M <= 24, "m-tiles");
+constexpr int K1S = K1 + 8;
+constexpr int FUSED_SMEM =
+    (32 * K1S + 40 * KPAD + FXH * FXW * 4 + F1P * CPAD + F2M * 16 * CPAD) * (int)sizeof(__nv_bfloat16) +
+    64 * (int)sizeof(float);
+
+struct NetFusedArgs {
+  int B, H, W;
+  const float *x;
+  float in_scale;
+  const __nv_bfloat16 *w1, *w2, *w3;
+  const float *b1, *b2, *b3;
+  __nv_bfloat16 *h1, *h2;
+  float *y;
+};
+
+// two n-tiles' B fragments of one k-step: rows n of the weights w (stride ws)
+__device__ __forceinline__ void b_frags(const __nv_bfloat16 *w, int ws, int n0, int k, int lane,
+                                        unsigned b[4]) {
+  const int mi = lane >> 3, mr = lane & 7;
+  ldsm_x4(smem_u32(&w[(n0 + (mi >> 1) * 8 + mr) * ws + k + (mi & 1) * 8]), b[0], b[1], b[2], b[3]);
+}
+// bias, ReLU and rounding of one m-tile's 32 channels into a shared activation
+// tile (zero outside the image; a tile well inside asks no pixel)
+__device__ __forceinline__ void put_hidden(const float acc[4][4], const float *bias, __nv_bfloat16 *s,
+                                           int p0, int width, bool inside, int i0, int j0, int H,
+                                           int W, int lane) {
+  unsigned keep[2] = {~0u, ~0u};
+  if (!inside) {
+#pragma unroll
+    for (int hh = 0; hh < 2; hh++) {
+      const int p = p0 + (lane >> 2) + hh * 8, gi = i0 + p / width, gj = j0 + p % width;
+      keep[hh] = gi >= 0 && gi < H && gj >= 0 && gj < W ? ~0u : 0u;
+    }
+  }
+  unsigned v[2][4];
+#pragma unroll
+  for (int nt = 0; nt < 4; nt++) {
+    const float2 b = *reinterpret_cast<const float2 *>(bias + nt * 8 + (lane & 3) * 2);
+#pragma unroll
+    for (int hh = 0; hh < 2; hh++) {
+      // the rounding keeps the sign, so the maximum may follow it
+      const float2 r = __fadd2_rn(make_float2(acc[nt][hh * 2], acc[nt][hh * 2 + 1]), b);
+      const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(r.x, r.y), __floats2bfloat162_rn(0.f, 0.f));
+      v[hh][nt] = *reinterpret_cast<const unsigned *>(&h) & keep[hh];
+    }
+  }
+  const unsigned at = smem_u32(s + (p0 + (lane & 7)) * CPAD + (lane >> 3) * 8);
+#pragma unroll
+  for (int hh = 0; hh < 2; hh++)
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(
+                     at + hh * 8 * CPAD * 2),
+                 "r"(v[hh][0]), "r"(v[hh][1]), "r"(v[hh][2]), "r"(v[hh][3])
+                 : "memory");
+}
+// the tile's own pixels of a shared activation (ring r, width w) to global memory
+__device__ __forceinline__ void store_hidden(const __nv_bfloat16 *s, int r, int w, __nv_bfloat16 *h,
+                                             int b, int i0, int j0, int H, int W, int tid) {
+  const int q = tid & 3, j = (tid >> 2) & 31, i = tid >> 7;
+  if (j0 + j >= W) return;
+  const uint4 *from = reinterpret_cast<const uint4 *>(s + ((i + r) * w + j + r) * CPAD) + q;
+  uint4 *to = reinterpret_cast<uint4 *>(h + (((size_t)b * H + i0 + i) * W + j0 + j) * CH) + q;
+#pragma unroll
+  for (int k = 0; k < NET_TH / 2; k++)
+    if (i0 + i + 2 * k < H) to[(size_t)k * 2 * W * (CH / 8)] = from[k * 2 * w * (CPAD / 8)];
+}
+// input pixels of tile (b, i0, j0): loads, and rounded stores
+struct InPixels {
+  float v[3][3];
+  __device__ __forceinline__ void load(const NetFusedArgs &a, int b, int i0, int j0, int tid) {
+    const long long hw = (long long)a.H * a.W;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const int e = tid + k * 256, gi = i0 + e / FXW - 3, gj = j0 + e % FXW - 3;
+      const bool in = e < FXH * FXW && gi >= 0 && gi < a.H && gj >= 0 && gj < a.W;
+      const float *q = a.x + 3 * b * hw + (long long)gi * a.W + gj;
+#pragma unroll
+      for (int c = 0; c < 3; c++) v[k][c] = in ? q[c * hw] : 0.f;
+    }
+  }
+  __device__ __forceinline__ void store(const NetFusedArgs &a, __nv_bfloat16 *s, int tid) const {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const int e = tid + k * 256;
+      if (e >= FXH * FXW) continue;
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(v[k][0] * a.in_scale, v[k][1] * a.in_scale);
+      const __nv_bfloat162 hi = __floats2bfloat162_rn(v[k][2] * a.in_scale, 0.f);
+      uint2 u;
+      u.x = *reinterpret_cast<const unsigned *>(&lo);
+      u.y = *reinterpret_cast<const unsigned *>(&hi);
+      *reinterpret_cast<uint2 *>(&s[e * 4]) = u;
+    }
+  }
+};
+
+__global__ void __launch_bounds__(256, 2) k_net_fused(NetFusedArgs a) {
+  extern __shared__ __align__(16) __nv_bfloat16 fs[];
+  __nv_bfloat16 *const s_w1 = fs, *const s_w2 = s_w1 + 32 * K1S, *const s_w3 = s_w2 + 32 * KPAD;
+  __nv_bfloat16 *const s_h1 = s_w3 + 8 * KPAD, *const s_h2 = s_h1 + F1P * CPAD;
+  __nv_bfloat16 *const s_x = s_h2 + F2M * 16 * CPAD;
+  float *const s_b = reinterpret_cast<float *>(s_x + FXH * FXW * 4);   // b1, b2
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, H = a.H, W = a.W;
+  const int mi = lane >> 3, mr = lane & 7, tig = lane & 3, g = lane >> 2;
+  for (int e = tid; e < 32 * K1 / 8; e += 256)
+    *reinterpret_cast<uint4 *>(&s_w1[e / (K1 / 8) * K1S + e % (K1 / 8) * 8]) =
+        reinterpret_cast<const uint4 *>(a.w1)[e];
+  for (int e = tid; e < 40 * KH / 8; e += 256) {      // w2 and w3 (32 and 8 rows)
+    const uint4 v = e < 32 * KH / 8 ? reinterpret_cast<const uint4 *>(a.w2)[e]
+                                    : reinterpret_cast<const uint4 *>(a.w3)[e - 32 * KH / 8];
+    *reinterpret_cast<uint4 *>(&s_w2[e / (KH / 8) * KPAD + e % (KH / 8) * 8]) = v;
+  }
+  if (tid < 64) s_b[tid] = tid < 32 ? a.b1[tid] : a.b2[tid - 32];
+  // input offsets of this lane's eight k pairs of the first layer; k >= 27 reads
+  // the zero that pads a pixel
+  int koff[2][2][2];
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const int k = (q >> 2) * 16 + ((q >> 1) & 1) * 8 + tig * 2 + (q & 1), t = k / 3;
+    koff[q >> 2][(q >> 1) & 1][q & 1] = k < 27 ? ((t / 3) * FXW + t % 3) * 4 + k % 3 : 3;
+  }
+  const int tw = (W + NET_TW - 1) / NET_TW, th = (H + NET_TH - 1) / NET_TH;
+  const long long tiles = (long long)a.B * tw * th, hw = (long long)H * W;
+  // tile t of batch b at (i0, j0)
+  auto tile = [&](long long t, int &b, int &i0, int &j0) {
+    b = (int)(t / (tw * th));
+    const int r = (int)(t - (long long)b * tw * th);
+    i0 = r / tw * NET_TH;
+    j0 = (r - r / tw * tw) * NET_TW;
+  };
+  int b, i0, j0;
+  tile(blockIdx.x, b, i0, j0);
+  InPixels in;
+  in.load(a, b, i0, j0, tid);
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    in.store(a, s_x, tid);
+    __syncthreads();
+    const bool inside = i0 >= 2 && j0 >= 2 && i0 + NET_TH + 2 <= H && j0 + NET_TW + 2 <= W;
+    // first activation on 12 x 36 pixels
+    const unsigned short *const xs = reinterpret_cast<const unsigned short *>(s_x);
+    unsigned wf[2][2][4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) b_frags(s_w1, K1S, (q & 1) * 16, (q >> 1) * 16, lane, wf[q >> 1][q & 1]);
+#pragma unroll 2
+    for (int mt = warp; mt < F1M; mt += 8) {
+      float acc[4][4];
+#pragma unroll
+      for (int nt = 0; nt < 4; nt++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[nt][q] = 0.f;
+      const int pa = mt * 16 + g, pb = pa + 8;
+      const unsigned short *const xa = xs + (pa / F1W * FXW + pa % F1W) * 4;
+      const unsigned short *const xb = xs + (pb / F1W * FXW + pb % F1W) * 4;
+#pragma unroll
+      for (int ks = 0; ks < 2; ks++) {
+        unsigned af[4];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const int o0 = koff[ks][h][0], o1 = koff[ks][h][1];
+          af[2 * h] = xa[o0] | (unsigned)xa[o1] << 16;
+          af[2 * h + 1] = xb[o0] | (unsigned)xb[o1] << 16;
+        }
+#pragma unroll
+        for (int n2 = 0; n2 < 2; n2++) {
+          const unsigned *bf = wf[ks][n2];
+          mma_bf16(acc[2 * n2], af[0], af[1], af[2], af[3], bf[0], bf[1]);
+          mma_bf16(acc[2 * n2 + 1], af[0], af[1], af[2], af[3], bf[2], bf[3]);
+        }
+      }
+      put_hidden(acc, s_b, s_h1, mt * 16, F1W, inside, i0 - 2, j0 - 2, H, W, lane);
+    }
+    __syncthreads();
+    store_hidden(s_h1, 2, F1W, a.h1, b, i0, j0, H, W, tid);
+    // second activation on 10 x 34 pixels: m-tiles warp, warp + 8, warp + 16
+    {
+      float acc[3][4][4];
+      unsigned row[3];
+      const bool third = warp + 16 < F2M;
+#pragma unroll
+      for (int m = 0; m < 3; m++) {
+        int p = (warp + 8 * m) * 16 + mr + (mi & 1) * 8;
+        p = p < F2P ? p : F2P - 1;
+        row[m] = smem_u32(&s_h1[(p / F2W * F1W + p % F2W) * CPAD + (mi >> 1) * 8]);
+#pragma unroll
+        for (int nt = 0; nt < 4; nt++)
+#pragma unroll
+          for (int q = 0; q < 4; q++) acc[m][nt][q] = 0.f;
+      }
+#pragma unroll 1
+      for (int ty = 0; ty < 3; ty++)
+#pragma unroll
+        for (int q = 0; q < 6; q++) {      // the row's three taps, two k-steps each
+          const unsigned off = ((ty * F1W + (q >> 1)) * CPAD + (q & 1) * 16) * 2;
+          unsigned bf[2][4], af[4];
+          b_frags(s_w2, KPAD, 0, ty * 96 + q * 16, lane, bf[0]);
+          b_frags(s_w2, KPAD, 16, ty * 96 + q * 16, lane, bf[1]);
+#pragma unroll
+          for (int m = 0; m < 3; m++) {
+            if (m == 2 && !third) break;
+            ldsm_x4(row[m] + off, af[0], af[1], af[2], af[3]);
+#pragma unroll
+            for (int nt = 0; nt < 4; nt++)
+              mma_bf16(acc[m][nt], af[0], af[1], af[2], af[3], bf[nt >> 1][(nt & 1) * 2],
+                       bf[nt >> 1][(nt & 1) * 2 + 1]);
+          }
+        }
+#pragma unroll
+      for (int m = 0; m < 3; m++) {
+        if (m == 2 && !third) break;
+        put_hidden(acc[m], s_b + 32, s_h2, (warp + 8 * m) * 16, F2W, inside, i0 - 1, j0 - 1, H, W,
+                   lane);
+      }
+    }
+    __syncthreads();
+    store_hidden(s_h2, 1, F2W, a.h2, b, i0, j0, H, W, tid);
+    // the next tile's input is on its way during the output layer
+    const int ob = b, oi = i0 + (warp >> 1) * 2, oj = j0 + (warp & 1) * 16;
+    if (t + gridDim.x < tiles) {
+      tile(t + gridDim.x, b, i0, j0);
+      in.load(a, b, i0, j0, tid);
+    }
+    // output: two rows of 16 pixels a warp, which share the fragments of the
+    // two middle ones of the four rows that they read
+    float acc[2][4];
+    unsigned w3f[9][4];                  // both k-steps of each tap
+#pragma unroll
+    for (int m = 0; m < 2; m++)
+#pragma unroll
+      for (int q = 0; q < 4; q++) acc[m][q] = 0.f;
+#pragma unroll
+    for (int tap = 0; tap < 9; tap++)
+      ldsm_x4(smem_u32(&s_w3[mr * KPAD + tap * 32 + mi * 8]), w3f[tap][0], w3f[tap][1], w3f[tap][2],
+              w3f[tap][3]);
+    const unsigned base = smem_u32(
+        &s_h2[((warp >> 1) * 2 * F2W + (warp & 1) * 16 + mr + (mi & 1) * 8) * CPAD + (mi >> 1) * 8]);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+      for (int q = 0; q < 6; q++) {
+        unsigned af[4];
+        ldsm_x4(base + ((r * F2W + (q >> 1)) * CPAD + (q & 1) * 16) * 2, af[0], af[1], af[2], af[3]);
+#pragma unroll
+        for (int m = 0; m < 2; m++)
+          if (r >= m && r - m < 3) {
+            const unsigned *bf = w3f[(r - m) * 3 + (q >> 1)] + (q & 1) * 2;
+            mma_bf16(acc[m], af[0], af[1], af[2], af[3], bf[0], bf[1]);
+          }
+      }
+    if (tig < 2) {
+#pragma unroll
+      for (int m = 0; m < 2; m++)
+#pragma unroll
+        for (int hh = 0; hh < 2; hh++) {
+          const int gi = oi + m, gj = oj + g + hh * 8;
+          if (gi >= H || gj >= W) continue;
+          float *o = a.y + (3 * ob + 2 * tig) * hw + (long long)gi * W + gj;
+          o[0] = acc[m][hh * 2] + a.b3[2 * tig];
+          if (tig == 0) o[hw] = acc[m][hh * 2 + 1] + a.b3[1];
+        }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Parameter packing: FP32 master parameters (w[o][c][u][v] per layer, then
 // biases) -> BF16 matrices [n][k], k = tap*CIN + c (first layer: tap*3 + c,
 // padded to 32), rows beyond the output channels zero (last layer: 8 rows).
@@ -681,6 +961,7 @@ struct fvna_net {
   float *y = nullptr, *g3 = nullptr, *gh2 = nullptr;
   float *part = nullptr;                // the training kernels' partial sums
   int blocks[3] = {0, 0, 0};            // their persistent grids (layers 1, 2, 3)
+  int fused_blocks = 0;                 // the fused forward's
   double *loss = nullptr;
   long long *nin = nullptr;
   long long cap_pix = 0;  // capacity of the activation buffers (B*H*W)
@@ -716,6 +997,36 @@ int net_reserve(fvna_net *n, long long pix) {
   NCK(cudaMalloc(&n->g3, (size_t)pix * 3 * sizeof(float)));
   NCK(cudaMalloc(&n->gh2, (size_t)pix * CH * sizeof(float)));
   n->cap_pix = pix;
+  return FVNA_OK;
+}
+
+// forward of a batch of planes into the network's own activations
+int net_forward(fvna_net *n, int B, int H, int W, const float *x, float in_scale, float *y,
+                cudaStream_t s) {
+  const long long hw = (long long)H * W;
+  // a block's halo would read what another one has written
+  if (x < y + 3 * B * hw && y < x + 3 * B * hw) {
+    NCK(net_forward_launch(n, B, H, W, x, hw, W, 3 * hw, in_scale, y, hw, W, 3 * hw, 0, 1.f, n->h1,
+                           n->h2, s));
+    return FVNA_OK;
+  }
+  if (!n->fused_blocks) {
+    int dev = 0, sms = 0, occ = 0;
+    NCK(cudaGetDevice(&dev));
+    NCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NCK(cudaFuncSetAttribute(k_net_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM));
+    NCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_net_fused, 256, FUSED_SMEM));
+    n->fused_blocks = (occ > 0 ? occ : 1) * sms;
+  }
+  NetFusedArgs a;
+  a.B = B; a.H = H; a.W = W;
+  a.x = x; a.in_scale = in_scale; a.y = y;
+  a.w1 = n->w1; a.w2 = n->w2; a.w3 = n->w3;
+  a.b1 = n->params + NET_OFF_B1; a.b2 = n->params + NET_OFF_B2; a.b3 = n->params + NET_OFF_B3;
+  a.h1 = n->h1; a.h2 = n->h2;
+  const long long tiles = (long long)B * ((H + NET_TH - 1) / NET_TH) * ((W + NET_TW - 1) / NET_TW);
+  k_net_fused<<<(int)(tiles < n->fused_blocks ? tiles : n->fused_blocks), 256, FUSED_SMEM, s>>>(a);
+  NCK(cudaGetLastError());
   return FVNA_OK;
 }
 
@@ -843,8 +1154,8 @@ int fvna_net_forward(fvna_net *n, int B, int H, int W, const float *x, float in_
   int rc = net_reserve(n, (long long)B * H * W);
   if (rc != FVNA_OK) return rc;
   long long hw = (long long)H * W;
-  NCK(net_forward_launch(n, B, H, W, x, hw, W, 3 * hw, in_scale, y, hw, W, 3 * hw, 0, 1.f, n->h1,
-                         n->h2, s));
+  rc = net_forward(n, B, H, W, x, in_scale, y, s);
+  if (rc != FVNA_OK) return rc;
   size_t hb = (size_t)B * hw * CH * sizeof(__nv_bfloat16);
   if (h1_out) NCK(cudaMemcpyAsync(h1_out, n->h1, hb, cudaMemcpyDeviceToDevice, s));
   if (h2_out) NCK(cudaMemcpyAsync(h2_out, n->h2, hb, cudaMemcpyDeviceToDevice, s));
@@ -887,8 +1198,8 @@ int fvna_net_train_step(fvna_net *n, int B, int H, int W, const float *x, float 
   int rc = net_reserve(n, (long long)B * H * W);
   if (rc != FVNA_OK) return rc;
   long long hw = (long long)H * W;
-  NCK(net_forward_launch(n, B, H, W, x, hw, W, 3 * hw, in_scale, n->y, hw, W, 3 * hw, 0, 1.f,
-                         n->h1, n->h2, s));
+  rc = net_forward(n, B, H, W, x, in_scale, n->y, s);
+  if (rc != FVNA_OK) return rc;
   NCK(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
   k_net_count<<<1, 32, 0, s>>>(B, H, W, margin, edges, n->nin);
   const long long px = (hw + 255) / 256;
