@@ -1,7 +1,7 @@
 // fvna_device.cuh -- device code of the finite-volume step (arXiv 1311.3004,
-// section 3): Roe solver, limited corrections, the line marcher shared by the
-// two sweeps, border handling, and the sweep kernels.  Included by one
-// translation unit per precision:
+// section 3): the analytic borders, and the Roe solver and fluxes of the
+// kernels outside the sweeps (first speeds, border fluxes, the Riemann entry
+// point).  Included by one translation unit per precision:
 //   fvna_fp64.cu  (binary64, compiled with -fmad=false so that every product
 //                  and sum rounds as written: the formulas below are evaluated
 //                  in the same order as the paper's definitions are written),
@@ -295,66 +295,5 @@ __device__ __forceinline__ void flux_data(const Iface<T> &I, const Iface<T> &Lf,
   o.F[1] = T(0.5) * (coef0 * I.W0[1] + coef1 * I.W1[1]);
   o.F[2] = T(0.5) * (coef0 * I.W0[2] + coef1 * I.W1[2] + coef2 * I.W2);
 }
-
-// Cell update of eq. fv-hr.  binary64: evaluated as written.
-template <bool COMP>
-__device__ __forceinline__ double cell_update(const P64 &, double q, double am_r, double ap_l,
-                                              double F_r, double F_l, double lam) {
-  return q - lam * (am_r + ap_l) - lam * (F_r - F_l);
-}
-
-// binary32 with COMP: the two increments of eq. fv-hr (fluctuations and the
-// correction-flux difference) are added to the old value with error-free
-// two-sums (Knuth) and their rounding errors folded back once (Neumaier), so
-// the new value is rounded once from the exact sum of the two increments.
-// Without COMP the update is evaluated as written.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-  s = a + b;
-  float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-template <bool COMP>
-__device__ __forceinline__ float cell_update(const P32 &, float q, float am_r, float ap_l,
-                                             float F_r, float F_l, float lam) {
-  if (!COMP) return q - lam * (am_r + ap_l) - lam * (F_r - F_l);
-  float t1 = -lam * (am_r + ap_l);
-  float t2 = -lam * (F_r - F_l);
-  float s, e1, e2;
-  two_sum(q, t1, s, e1);
-  two_sum(s, t2, s, e2);
-  return s + (e1 + e2);
-}
-
-// ---------------------------------------------------------------------------
-// Line marcher: cells of one line are pushed in order; once four cells are
-// in, every push updates the cell two behind (eq. fv-hr), using the
-// interfaces on its two faces and their neighbours for the limiter.
-// ---------------------------------------------------------------------------
-template <class P> struct Marcher {
-  typedef typename P::T T;
-  T beta2, lam;
-  int lim;
-  // cells c-2, c-1 (old values) and z of c-1
-  T a2_, b2_, c2_, a1_, b1_, c1_, zb1, zc1;
-  Iface<T> Im2, Im1;          // interfaces c-2, c-1 (interface k lies between cells k-1, k)
-  T ap_l[3], F_l[3];          // flux data of interface c-2 (left face of cell c-2)
-  bool nonreal;
-
-  __device__ __forceinline__ void first(T a, T b, T c) {
-    T r = P::rq1(a);
-    a1_ = a; b1_ = b; c1_ = c;
-    zb1 = b * r; zc1 = c * r;
-    nonreal = false;
-  }
-  // push cell 1..: compute the interface with the previous cell
-  __device__ __forceinline__ void iface(T a, T b, T c, Iface<T> &I) {
-    T r = P::rq1(a);
-    T zb = b * r, zc = c * r;
-    nonreal |= roe(P(), beta2, a1_, b1_, c1_, zb1, zc1, a, b, c, zb, zc, I);
-    a2_ = a1_; b2_ = b1_; c2_ = c1_;
-    a1_ = a; b1_ = b; c1_ = c;
-    zb1 = zb; zc1 = zc;
-  }
-};
 
 }  // namespace fvna
