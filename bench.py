@@ -263,7 +263,7 @@ _TRAFFIC_KEYS = [
     (r"k_sweep_x64<", "k_sweep_x_fp64"),
     (r"k_sweep_y64<", "k_sweep_y_fp64"),
 ]
-# the 3D kernels (k3_sweep_v serves the x2 and the x3 sweep: one figure for both)
+# the 3D kernels (k3_sweep_vp serves the x2 and the x3 sweep: one figure for both)
 _TRAFFIC_KEYS3 = [
     (r"k3_sweep_xp<", "k3_sweep_x_fp32"), (r"k3_sweep_vp<", "k3_sweep_v_fp32"),
     (r"k3_source<float", "k3_source_fp32"), (r"k3_sweep64<", "k3_sweep_x_fp64"),
