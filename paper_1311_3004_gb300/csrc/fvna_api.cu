@@ -942,11 +942,12 @@ int fvna_set_correction(fvna_ctx *c, fvna_net *net, float in_scale, float out_sc
   if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
   if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
   // the correction runs between the x2 sweep and the step end, so with a
-  // network the step end is its own launch again
+  // network the step end is its own launch again (a Strang step, which takes
+  // no network, ends after its second x1 sweep: never in the x2 sweep)
   c->kernels_per_step += (net ? 3 : 0) - (c->net ? 3 : 0);
   if (c->cfg.precision == FVNA_FP32_PERT) {
     c->kernels_per_step += (net ? 1 : 0) - (c->net ? 1 : 0);
-    c->args_y.fold_advance = net ? 0 : 1;
+    c->args_y.fold_advance = net || c->cfg.splitting == FVNA_SPLIT_STRANG ? 0 : 1;
   }
   c->net = net;
   c->net_in = in_scale;
