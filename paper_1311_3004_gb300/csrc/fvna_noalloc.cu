@@ -11,7 +11,8 @@
 // __device__ array of fixed size, reserved when the library is loaded and
 // held by every GPU that loads it until the process exits.
 //
-// The step launches the same k_sweep_x64 / k_sweep_y64 pair as fvna_step, so
+// The step launches the same pair as fvna_step (k_sweep_x64, then k_sweep_y64
+// or k_sweep_yl64 by the size), so
 // its results are identical.  The kernels work their tiles out from the
 // domain's size (one domain needs no tile list).
 #include <cuda_runtime.h>
@@ -49,8 +50,13 @@ int setup_device(int dev) {
   if (g_addr[dev]) return FVNA_OK;
   void *p = nullptr;
   if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || !p) return FVNA_ERR_CUDA;
-  for (int lim = 0; lim < 3; lim++)
+  // every sweep kernel a call can launch, whatever its limiter and size: the
+  // occupancy queries load them all, so that no later call takes device
+  // memory for code
+  for (int lim = 0; lim < 3; lim++) {
     if (prepare_kernels_fp64(0, lim, 0) != cudaSuccess) return FVNA_ERR_CUDA;
+    occupancy_y_fp64(lim, 0);
+  }
   if (cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return FVNA_ERR_CUDA;
   g_addr[dev] = p;
