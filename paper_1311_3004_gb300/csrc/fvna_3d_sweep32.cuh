@@ -179,7 +179,9 @@ __device__ __forceinline__ void flux4p(const FaceP &I, const FaceP &Lf, const Fa
 
 // Statistics of a march or segment: max |s| (NaN-propagating), the smallest
 // c^2 - 1 over the faces of the non-real test, and what tells whether SPEC
-// held: the smallest min(s0, -s1) and the largest |c^2 - 1|.
+// held: the smallest min(s0, -s1) and the largest |c^2 - 1|, a NaN being
+// larger than any (it stands for what it hides: another face of the lane,
+// on the other line of its pair, may need the general split).
 struct Stat {
   float smax, dmin, subs, dmax;
   __device__ __forceinline__ void init() { smax = 0.f; dmin = 0.f; subs = 1.f; dmax = 0.f; }
@@ -196,7 +198,7 @@ struct Stat {
     if (ny) dmin = fminf(dmin, dm.y);
   }
   __device__ __forceinline__ bool spec_held() const {
-    return !__any_sync(0xffffffffu, subs <= 0.f || dmax >= x2::DM_SERIES);
+    return !__any_sync(0xffffffffu, subs <= 0.f || !(dmax < x2::DM_SERIES));
   }
   __device__ __forceinline__ void merge(const Stat &o) {
     smax = x2::max3_abs_nan(smax, o.smax, 0.f);
