@@ -100,9 +100,9 @@ typedef struct fvna_config {
   int tile_x;           /* x1-sweep tile width: binary32 16, 32 or 64 cells per warp row, or 60
                            (the x1 sweep with the lanes along x1); binary64 16 or 32 (one cell
                            per lane) or 64 (two); 0 = default (picked from the domain sizes) */
-  int tile_y;           /* x2-sweep tile height (rows per warp); 0 = default (binary64 picked
-                           from the domain sizes, binary32 10: 16 marched rows, two whole
-                           8-row chunks) */
+  int tile_y;           /* x2-sweep tile height (rows per warp); 0 = default (picked from the
+                           domain sizes; binary32 2, 10, 18, 26, 34 or 42: the marched rows,
+                           six more, are whole 8-row chunks) */
   int compensated;      /* FVNA_FP32_PERT: 0 = the increments of eq. fv-hr summed and added
                            to the state in one fused multiply-add (one rounding of the sum;
                            the default), 1 = the state and the two increments summed with

@@ -338,13 +338,15 @@ static double tile_cost(long long tiles, int sms, int per_tile, int want) {
   double fill = std::min(1.0, (double)tiles / sms / want);
   return per_sm * per_tile / fill;
 }
+// Times of the two forms in us, fitted to domains of 4,000 to 2 million cells:
+// the marched tiles 8.5 + 0.078 of their cost; segments with the lanes along x1
+// (two rows of 60 cells) 9 and 0.75 a thousand, 1.2 those at an x1 border.  The
+// segments leave no lane a line to march, so compact domains take them (1024^2
+// cells 16.0 against 17.4 to 22 for the marched tiles, 257 x 129 9.3 against
+// 10.3); a narrow domain fills no segment (1 x 400,000 cells 268 against 86, 8 x
+// 40,000 32 against 21, 64 x 16,384 28 against 20).  From two million cells on
+// the marched tiles, which the fit leaves out (2048^2 34.4 against 38.5).
 static int pick_tile_x32(int n, const fvna_domain *d, int sms) {
-  // below two million cells the segments with the lanes along x1, which leave
-  // no lane a line to march (1024^2 cells 16.5 us against 17.4 to 22 for the
-  // marched tiles, 257 x 129 9.3 against 10.3; at 2048^2 38.5 against 34.4)
-  long long cells = 0;
-  for (int k = 0; k < n; k++) cells += (long long)d[k].nx * d[k].ny;
-  if (cells < 2000000) return X32H_TILE;
   int best = 64;
   double best_cost = 1e300;
   for (int tx : {64, 32, 16}) {
@@ -355,23 +357,34 @@ static int pick_tile_x32(int n, const fvna_domain *d, int sms) {
     double c = tile_cost(T, sms, sw + 4, 7);
     if (c < best_cost) { best_cost = c; best = tx; }
   }
-  return best;
+  double cells = 0.0, segments = 9.0;
+  for (int k = 0; k < n; k++) {
+    const int cols = (d[k].nx + X32H_TILE - 1) / X32H_TILE, border = std::min(cols, 2);
+    cells += d[k].nx * (double)d[k].ny;
+    segments += (d[k].ny + 1) / 2 * (1.2e-3 * border + 0.75e-3 * (cols - border));
+  }
+  return cells < 2e6 && segments <= 8.5 + 0.078 * best_cost ? X32H_TILE : best;
 }
 // x2 sweep: a tile of ty rows marches ty + 6, so the work falls with the
 // height as (ty + 6)/ty while the last tiles, which nothing overlaps, take
 // ty + 6 steps.  Measured, the sweep takes about 5.5 us per million marched
-// cells and 0.9 us per step of its last tiles; heights whose marched rows fill
-// whole 8-row chunks.  (us for ty = 10, 18, 26, 34, 42: 2048^2 49.7, 53, 62,
-// 74, 82; 3000^2 90, 82, 80, 93, 102; 4096^2 154, 136, 130, 130, 130; 39
-// million cells in 48 domains 385, 341, 324, 320, 320.  257 x 129: 25
-// at 10 and 16 at 2.)
+// cells (60 a row of a tile, whatever the domain fills of them; twice as long
+// in a tile that holds both x1 borders) and 0.95 us per step of its last tiles;
+// heights whose marched rows fill whole 8-row chunks.  (us for ty = 10, 18, 26,
+// 34, 42: 2048^2 49.7, 53, 62, 74, 82; 3000^2 90, 82, 80, 93, 102; 4096^2 154,
+// 136, 130, 130, 130; 39 million cells in 48 domains 385, 341, 324, 320, 320; 1 x
+// 400,000 414, 358, 342, 336, 332, and 930 at 2.  At 2 and 10: 257 x 129 16 and
+// 25, 613 x 861 27 and 33, 8 x 40,000 107 and 61.)
 static int pick_tile_y32(int n, const fvna_domain *d) {
-  double cells = 0.0;
-  for (int k = 0; k < n; k++) cells += 1e-6 * d[k].nx * (double)d[k].ny;
   int best = 10;
   double best_cost = 1e300;
   for (int ty : {2, 10, 18, 26, 34, 42}) {
-    const double c = 5.5 * cells * (ty + 6) / ty + 0.9 * (ty + 6);
+    double marched = 0.0;
+    for (int k = 0; k < n; k++) {
+      const int cols = (d[k].nx + Y32_COLS - 1) / Y32_COLS;
+      marched += (cols == 1 ? 2.0 : cols) * ((d[k].ny + ty - 1) / ty) * (ty + 6) * (1e-6 * Y32_COLS);
+    }
+    const double c = 5.5 * marched + 0.95 * (ty + 6);
     if (c < best_cost) { best_cost = c; best = ty; }
   }
   return best;

@@ -1,0 +1,55 @@
+"""The tile shapes the library picks for itself: a step of a narrow binary32
+domain takes no longer in the picked shapes than in shapes given by hand.
+Times are the shortest of several runs of one step graph; the margin of 1.25 is far above
+their scatter (a few percent) and far below what a wrong shape costs (1.6 and
+more in these sizes)."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1311_3004_gb300 import fvna
+from paper_1311_3004_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+MARGIN = 1.25
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1311_3004_gb300 import build
+    build.build()
+
+
+def _config(precision, tile_x=0, tile_y=0):
+    return fvna.make_config(precision=precision, beta=3.5, delta=1e-4, dx=1.0 / 40, nu_w=0.9,
+                            steps_per_graph=16, tile_x=tile_x, tile_y=tile_y)
+
+
+def _state(nx, ny):
+    q = wl.ambient(nx, ny)
+    q[0] += 1e-3 * np.cos(0.05 * np.arange(ny))[:, None] * np.cos(0.05 * np.arange(nx))
+    return q
+
+
+def _time(cfg, nx, ny, q):
+    torch = pytest.importorskip("torch")
+    s = fvna.Solver(cfg, [fvna.make_domain(nx, ny)], [q])
+    s.run(max_steps=16)
+    best = 1e9
+    for _ in range(9):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        s.run(max_steps=16)
+        best = min(best, time.perf_counter() - t0)
+    s.close()
+    return best
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 400000), (4, 400000), (8, 40000)])
+def test_narrow_domains_fp32(nx, ny):
+    q = _state(nx, ny)
+    picked = _time(_config(fvna.FP32_PERT), nx, ny, q)
+    given = min(_time(_config(fvna.FP32_PERT, 16, ty), nx, ny, q) for ty in (10, 18))
+    assert picked <= MARGIN * given, (picked, given)
