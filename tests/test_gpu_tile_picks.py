@@ -1,8 +1,9 @@
 """The tile shapes the library picks for itself: a step of a narrow binary32
-domain takes no longer in the picked shapes than in shapes given by hand.
-Times are the shortest of several runs of one step graph; the margin of 1.25 is far above
-their scatter (a few percent) and far below what a wrong shape costs (1.6 and
-more in these sizes)."""
+domain takes no longer in the picked shapes than in shapes given by hand, and
+what fvna_autotune returns is no slower than the picked shapes.  Times are the
+shortest of several runs of one step graph; the margin of 1.25 is far above
+their scatter (a few percent) and below what a wrong shape costs (1.4 and more in
+these sizes)."""
 import time
 
 import numpy as np
@@ -53,3 +54,13 @@ def test_narrow_domains_fp32(nx, ny):
     picked = _time(_config(fvna.FP32_PERT), nx, ny, q)
     given = min(_time(_config(fvna.FP32_PERT, 16, ty), nx, ny, q) for ty in (10, 18))
     assert picked <= MARGIN * given, (picked, given)
+
+
+@pytest.mark.parametrize("precision,nx,ny", [(fvna.FP64, 512, 8), (fvna.FP64, 300, 300),
+                                             (fvna.FP32_PERT, 61, 61)])
+def test_tuned_no_slower_than_picked(precision, nx, ny):
+    q = _state(nx, ny)
+    best, ms = fvna.autotune(_config(precision), [fvna.make_domain(nx, ny)], [q], trial_steps=16)
+    assert ms > 0 and best.steps_per_graph == 16
+    tuned, picked = _time(best, nx, ny, q), _time(_config(precision), nx, ny, q)
+    assert tuned <= MARGIN * picked, (tuned, picked, best.tile_x, best.tile_y)
