@@ -224,7 +224,7 @@ class ClockSampler:
 _SWEEP_SOURCES = ["fvna_api.cu", "fvna_device.cuh", "fvna_face64.cuh", "fvna_fp32.cu",
                   "fvna_fp64.cu", "fvna_int64f.cuh", "fvna_sweeps64.cuh",
                   "fvna_launch.h", "fvna_precision.inc", "fvna_step.cuh", "fvna_sweeps.cuh",
-                  "fvna_sweeps32.cuh", "fvna_types.h", "fvna_x2.cuh"]
+                  "fvna_sweeps32.cuh", "fvna_types.h", "fvna_x2.cuh", "fvna_xh.cuh"]
 
 
 _SWEEP3_SOURCES = ["fvna_3d.cuh", "fvna_3d.inc", "fvna_3d_sweep32.cuh", "fvna_3d_sweep64.cuh",
@@ -254,19 +254,25 @@ def ncu_traffic(kernel_key: str, files=None):
     return e.get("dram_bytes_per_launch")
 
 
-# sweep kernels of the timed step, by the demangled names ncu prints: the
-# binary32 x2 sweep's second kernel (REDO = true) belongs to the x2 sweep
-# (ncu prints template arguments without namespaces and bools as 0 / 1)
+# sweep kernels of the timed step, by the demangled names ncu prints, one key a
+# sweep whichever kernel the size runs (k_sweep_x32h and k_sweep_yl64 are those of
+# small domains): the binary32 x2 sweep's second kernel (REDO = true) belongs to
+# the x2 sweep (ncu prints template arguments without namespaces and bools as 0 / 1)
 _TRAFFIC_KEYS = [
-    (r"k_sweep_x32<", "k_sweep_x_fp32"),
+    (r"k_sweep_x32h?<", "k_sweep_x_fp32"),
     (r"k_sweep_y32<", "k_sweep_y_fp32"),
     (r"k_sweep_x64<", "k_sweep_x_fp64"),
-    (r"k_sweep_y64<", "k_sweep_y_fp64"),
+    (r"k_sweep_yl?64<", "k_sweep_y_fp64"),
 ]
-# the 3D kernels (k3_sweep_vp serves the x2 and the x3 sweep: one figure for both)
+# kernels of a 3D step in the order of fvna3_step_timed; a kernel that serves
+# several sweeps has one figure for them
+_KERNELS3 = {
+    "fp32": ["k3_sweep_xp", "k3_sweep_vp (x2)", "k3_sweep_vp (x3)", "k3_source"],
+    "fp64": ["k3_sweep64 (x1)", "k3_sweep64 (x2)", "k3_sweep64 (x3)", "k3_source"],
+}
 _TRAFFIC_KEYS3 = [
-    (r"k3_sweep_xp<", "k3_sweep_x_fp32"), (r"k3_sweep_vp<", "k3_sweep_v_fp32"),
-    (r"k3_source<float", "k3_source_fp32"), (r"k3_sweep64<", "k3_sweep_x_fp64"),
+    (r"k3_sweep_xp<", "k3_sweep_xp_fp32"), (r"k3_sweep_vp<", "k3_sweep_vp_fp32"),
+    (r"k3_source<float", "k3_source_fp32"), (r"k3_sweep64<", "k3_sweep64_fp64"),
     (r"k3_source<double", "k3_source_fp64"),
 ]
 
@@ -878,7 +884,7 @@ def run_gaussian3d(args):
             per = np.array(per)
             esz = 4 if prec == fvna.FP32_PERT else 8
             alg = 2 * 4 * esz * cells            # one sweep reads and writes the four fields
-            kn = ["k3_sweep_x", "k3_sweep_v (x2)", "k3_sweep_v (x3)", "k3_source"]
+            kn = _KERNELS3[name]
             avg = per[:, :4].mean(axis=0)
             k = int(np.argmax(avg))
             ach = alg / (avg[k] * 1e-3) / 1e9
