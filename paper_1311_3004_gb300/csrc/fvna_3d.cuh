@@ -197,22 +197,6 @@ __device__ __forceinline__ unsigned long long speed_bits(float s) {
   if (a != a) return 0x7ff8000000000000ull;
   return speed_bits((double)a);
 }
-// Running max |s| of a march in the precision's own bits (binary32: 32-bit
-// patterns, every NaN above +inf), widened to the binary64 pattern of the
-// domain scalars once per march.
-template <class T> struct Speed;
-template <> struct Speed<double> {
-  typedef unsigned long long B;
-  __device__ static B bits(double s) { return speed_bits(s); }
-  __device__ static unsigned long long wide(B b) { return b; }
-};
-template <> struct Speed<float> {
-  typedef unsigned B;
-  __device__ static B bits(float s) { return __float_as_uint(fabsf(s)); }
-  __device__ static unsigned long long wide(B b) {
-    return b > 0x7f800000u ? 0x7ff8000000000000ull : speed_bits((double)__uint_as_float(b));
-  }
-};
 
 // warp-wide statistics of a march into the scalars
 __device__ __forceinline__ void flush_stats(Scal3 *S, unsigned long long smax, bool nonreal) {
@@ -287,7 +271,9 @@ template <class T> __device__ __forceinline__ void zof3(const T q[4], T z[3]) {
 // ahead) is loaded while the current plane is formed.  Threads of a tile
 // that overhangs the domain form ghost or clamped cells and store nothing.
 constexpr int SRC3_TX = 32, SRC3_TY = 8;
-constexpr int SRC3_BLOCKS = 608;   // blocks wanted before chunks are shortened: four an SM
+// blocks wanted before chunks are shortened: four for each of 152 SMs, in both
+// precisions (64^3 in binary64, two resident blocks an SM: 80 us in chunks of 16, 33 now)
+constexpr int SRC3_BLOCKS = 608;
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 2) k3_source(Args3 A) {
   Scal3 *S = A.S;

@@ -10,8 +10,13 @@
 //                 tile of TY cells and two halo cells at each end, one
 //                 coalesced 8-byte load per field and cell.
 //
-// What bounds them is instruction issue.  One line a lane took 488 (x1) and 331
-// (x2, x3) instructions a cell; a pair shares them.  As in the 2D sweeps every
+// What bounds them is issue and latency together, not memory (128^3: 15 % of the
+// DRAM rate).  x1: 14 warps an SM issue in 58 % of the cycles and wait for
+// their loads (1.5 warps an issue) and for results (1.1).  x2, x3: 168 registers
+// leave 11 warps an SM, which issue in 40 % and wait for the next cell's loads
+// (3.3).  The MC forms spill a little (52 and 136 bytes of loads).  One line a
+// lane took 488 (x1) and 331 (x2, x3) instructions a cell; a pair shares them: 275
+// and 179 a cell (128-cell rows: three segments of 60).  As in the 2D sweeps every
 // face is first taken as subsonic with 1/c from its series (no branch a face,
 // a shorter chain), and a segment or tile that met another face is done again
 // with the general split.  Tile heights are picked for whole rounds of the
@@ -205,7 +210,7 @@ struct Stat {
     dmin = fminf(dmin, o.dmin);
   }
   __device__ __forceinline__ void flush(Scal3 *S) const {
-    flush_stats(S, Speed<float>::wide(Speed<float>::bits(smax)), dmin < -1.f);
+    flush_stats(S, speed_bits(smax), dmin < -1.f);
   }
 };
 

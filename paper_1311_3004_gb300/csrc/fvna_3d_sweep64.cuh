@@ -6,8 +6,11 @@
 // f64::lanes_step.  Along x1 a warp's loads are one coalesced run; along x2
 // and x3 the lanes are rows or planes apart, and the four warps of a block sit
 // on neighbouring x1 columns, so that they share the 32-byte sectors the lanes
-// touch.  The sweep is bound by the binary64 unit (fvna_face64.cuh), not by
-// these loads: 256^3 cells move 1.07 GB a sweep, a sixth of a millisecond.
+// touch.  The sweep is bound by the binary64 unit (fvna_face64.cuh; 128^3: busy
+// for 89, 89 and 87 % of its cycles), not by these loads: 256^3 cells move 1.07
+// GB a sweep, a sixth of a millisecond.  A direction of a few cells fills few of
+// a segment's lanes: the x3 sweep of 256 x 256 x 3 takes 434 us, twice what
+// marched columns took, its whole step 574 against 1223.
 #pragma once
 
 #include "fvna_3d.cuh"

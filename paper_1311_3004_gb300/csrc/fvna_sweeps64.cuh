@@ -12,8 +12,10 @@
 //                in shared memory (coalesced along the row), and the source is
 //                applied one row behind the sweep, with the x neighbours taken
 //                from the adjacent lanes by warp shuffles.  Twelve warps an SM
-//                with a few spilled registers are faster than sixteen or eight
-//                (2048 x 2048 cells: 1.04, 1.10, 1.37 ms).
+//                are faster than sixteen or eight (2048 x 2048 cells: 1.04,
+//                1.10, 1.37 ms), although the three forms of a step do not
+//                fit their 168 registers (MC limiter: 452 bytes of spill
+//                stores, 1,368 of spill loads; 9.7 M of 416 M instructions).
 //   k_sweep_yl64 the same for domains of fewer cells: the lanes along x2, a
 //                column of 32 rows at a time, and the block's warps on
 //                neighbouring columns, whose velocities meet in shared memory
@@ -23,9 +25,12 @@
 //                height; 512 x 8: 18 against 58).
 //
 // Both are bound by the binary64 unit, of which every SM quarter has its own
-// (64 cycles a warp instruction): what counts is how evenly the cells spread
-// over the quarters, and how few instructions a cell sends there
-// (fvna_face64.cuh).  The x1 sweep had the lanes on 32 rows and marched 36
+// (64 cycles a warp instruction; 2048 x 2048 cells: busy for 87 % of the
+// x1 sweep's cycles and 81 % of the x2 sweep's): what counts is how evenly the
+// cells spread over the quarters, and how few instructions a cell sends there
+// (fvna_face64.cuh).  The tiles are dealt in turn, so a warp with slower ones ends
+// the x2 sweep: a pulse's step takes 1.84 ms on a fresh state and 2.03 ms when
+// its precursor has spread.  The x1 sweep had the lanes on 32 rows and marched 36
 // cells in each: 512 x 8 cells were 16 warps of 36 steps, 0.5 ms, now 152
 // warps of one, 13 us.
 #pragma once

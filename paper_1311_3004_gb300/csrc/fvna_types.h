@@ -10,9 +10,8 @@ enum { LIM_MC = 0, LIM_NONE = 1, LIM_LW = 2 };
 // ST_TIMEOUT: a kernel gave up waiting for one of its own asynchronous copies
 enum { ST_NONREAL = 1, ST_CFL = 2, ST_NAN = 4, ST_TIMEOUT = 8 };
 
-// Halo widths: the x1 sweep reads 2 cells beyond its tile (the limiter looks
-// one interface upwind), the x2 sweep with the fused source reads 3.
-constexpr int HALO_X = 2;
+// Halo width of the x2 sweep with the fused source (a sweep alone reads 2 cells
+// beyond its tile, the limiter looking one interface upwind).
 constexpr int HALO_Y = 3;
 // Axisymmetric form: radial faces next to the axis that use the first-order
 // flux (r = 0 and r = dx).
