@@ -1004,12 +1004,6 @@ int net_reserve(fvna_net *n, long long pix) {
 int net_forward(fvna_net *n, int B, int H, int W, const float *x, float in_scale, float *y,
                 cudaStream_t s) {
   const long long hw = (long long)H * W;
-  // a block's halo would read what another one has written
-  if (x < y + 3 * B * hw && y < x + 3 * B * hw) {
-    NCK(net_forward_launch(n, B, H, W, x, hw, W, 3 * hw, in_scale, y, hw, W, 3 * hw, 0, 1.f, n->h1,
-                           n->h2, s));
-    return FVNA_OK;
-  }
   if (!n->fused_blocks) {
     int dev = 0, sms = 0, occ = 0;
     NCK(cudaGetDevice(&dev));
@@ -1018,13 +1012,27 @@ int net_forward(fvna_net *n, int B, int H, int W, const float *x, float in_scale
     NCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_net_fused, 256, FUSED_SMEM));
     n->fused_blocks = (occ > 0 ? occ : 1) * sms;
   }
+  const int th = (H + NET_TH - 1) / NET_TH;
+  const long long tiles = (long long)B * th * ((W + NET_TW - 1) / NET_TW);
+  // The layers one by one where the output overlaps the input (a block's halo
+  // would read what another one has written), and for many tiles with less than
+  // two fifths of their pixels in the image, where the fused kernel's rings cost
+  // more than its one pass saves (60,000 images of 1 x 1 1.38 ms against 1.57, 8,192 of
+  // 9 x 33 0.88 against 0.98; full tiles 0.33 against 0.27, half-full ones alike).
+  // A call of few tiles is three launches' latency against one's.
+  const bool overlap = x < y + 3 * B * hw && y < x + 3 * B * hw;
+  const bool sparse = tiles > n->fused_blocks && 5 * B * hw < 2 * tiles * NET_PIX;
+  if (overlap || (sparse && B <= 65535 && th <= 65535)) {   // (grid limits of the layers)
+    NCK(net_forward_launch(n, B, H, W, x, hw, W, 3 * hw, in_scale, y, hw, W, 3 * hw, 0, 1.f, n->h1,
+                           n->h2, s));
+    return FVNA_OK;
+  }
   NetFusedArgs a;
   a.B = B; a.H = H; a.W = W;
   a.x = x; a.in_scale = in_scale; a.y = y;
   a.w1 = n->w1; a.w2 = n->w2; a.w3 = n->w3;
   a.b1 = n->params + NET_OFF_B1; a.b2 = n->params + NET_OFF_B2; a.b3 = n->params + NET_OFF_B3;
   a.h1 = n->h1; a.h2 = n->h2;
-  const long long tiles = (long long)B * ((H + NET_TH - 1) / NET_TH) * ((W + NET_TW - 1) / NET_TW);
   k_net_fused<<<(int)(tiles < n->fused_blocks ? tiles : n->fused_blocks), 256, FUSED_SMEM, s>>>(a);
   NCK(cudaGetLastError());
   return FVNA_OK;
