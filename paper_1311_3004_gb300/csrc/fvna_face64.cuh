@@ -4,7 +4,12 @@
 //
 // Two forms of each, with the same results bit for bit (a zero's sign aside):
 //   *_general  every formula in the order of its definition on the binary64
-//              unit (the including units are compiled with -fmad=false);
+//              unit (the including units are compiled with -fmad=false; a sum
+//              is the fused multiply-add x 1 + y, a product x y + (-0), which
+//              round alike and are taken faster, see below).  2048 x 2048 cells
+//              wholly in this form (beta 6.3): x1 and x2 sweep 1.92 and 1.84 ms;
+//              2.35 and 2.14 with plain operations, a 0/0 a warp and no
+//              subsonic form; 1.76 and 2.23 in the kernels before these;
 //   *_fast     the same roundings with fewer instructions on that unit:
 //              reciprocals, quotients, roots and the products of the solver
 //              and of the limiter's sums run in integer arithmetic
@@ -126,10 +131,10 @@ template <int NT> struct Flux {
 
 // velocities z = (normal, transverse) / q1
 template <int NT>
-__device__ __forceinline__ void z_general(const double q[2 + NT], double z[1 + NT]) {
+__device__ __forceinline__ void z_general(const Unit &U, const double q[2 + NT], double z[1 + NT]) {
   const double r = 1.0 / q[0];
 #pragma unroll
-  for (int k = 0; k < 1 + NT; k++) z[k] = q[1 + k] * r;
+  for (int k = 0; k < 1 + NT; k++) z[k] = U.mul(q[1 + k], r);
 }
 template <int NT> __device__ __forceinline__ void z_fast(const Par &P, const double q[2 + NT], double z[1 + NT]) {
   const double r = int64f::rcp_mid(q[0]);
@@ -139,36 +144,38 @@ template <int NT> __device__ __forceinline__ void z_fast(const Par &P, const dou
 
 // Roe solver (section 3.2) of cells L and R; true if the radicand is negative.
 template <int NT>
-__device__ __forceinline__ bool face_general(double beta2, const double L[2 + NT],
+__device__ __forceinline__ bool face_general(const Par &P, const double L[2 + NT],
                                              const double zL[1 + NT], const double R[2 + NT],
                                              const double zR[1 + NT], Face<NT> &F) {
-  const double Z1 = 0.5 * (L[0] + R[0]);
-  const double Z2 = 0.5 * (zL[0] + zR[0]);
-  const double Phi = 1.0 + beta2 * (Z1 - 1.0);
+  const Unit &U = P.U;
+  const double Z1 = U.mul(0.5, U.add(L[0], R[0]));
+  const double Z2 = U.mul(0.5, U.add(zL[0], zR[0]));
+  const double Phi = U.add(U.mul(P.beta2, U.add(Z1, -1.0)), 1.0);
   const double rZ1 = 1.0 / Z1;
-  const double u = Z2 * rZ1;
-  const double D = u * u - 2.0 * Z2 * u + Phi;
+  const double u = U.mul(Z2, rZ1);
+  const double T2 = U.add(Z2, Z2);
+  const double D = U.add(U.sub(U.mul(u, u), U.mul(T2, u)), Phi);
   const bool nonreal = D < 0.0;
   const double c = sqrt(D);
-  F.s0 = u + c;
-  F.s1 = u - c;
+  F.s0 = U.add(u, c);
+  F.s1 = U.sub(u, c);
   F.u = u;
   const double rc = 1.0 / c;
-  const double h = 0.5 * rc;
-  const double d1 = R[0] - L[0];
-  const double d2 = R[1] - L[1];
-  F.a1 = (d2 - F.s1 * d1) * h;
-  F.a2 = (F.s0 * d1 - d2) * h;
-  F.w01 = F.a1 * F.s0;
-  F.w11 = F.a2 * F.s1;
+  const double h = U.mul(0.5, rc);
+  const double d1 = U.sub(R[0], L[0]);
+  const double d2 = U.sub(R[1], L[1]);
+  F.a1 = U.mul(U.sub(d2, U.mul(F.s1, d1)), h);
+  F.a2 = U.mul(U.sub(U.mul(F.s0, d1), d2), h);
+  F.w01 = U.mul(F.a1, F.s0);
+  F.w11 = U.mul(F.a2, F.s1);
 #pragma unroll
   for (int k = 0; k < NT; k++) {
-    const double v = (0.5 * (zL[1 + k] + zR[1 + k])) * rZ1;
-    const double r1 = v * (F.s0 - 2.0 * Z2) * rc;
-    const double r2 = v * (2.0 * Z2 - F.s1) * rc;
-    F.w0[k] = F.a1 * r1;
-    F.w1[k] = F.a2 * r2;
-    F.w2[k] = (R[2 + k] - L[2 + k]) - F.w0[k] - F.w1[k];
+    const double v = U.mul(U.mul(0.5, U.add(zL[1 + k], zR[1 + k])), rZ1);
+    const double r1 = U.mul(U.mul(v, U.sub(F.s0, T2)), rc);
+    const double r2 = U.mul(U.mul(v, U.sub(T2, F.s1)), rc);
+    F.w0[k] = U.mul(F.a1, r1);
+    F.w1[k] = U.mul(F.a2, r2);
+    F.w2[k] = U.sub(U.sub(U.sub(R[2 + k], L[2 + k]), F.w0[k]), F.w1[k]);
   }
   return nonreal;
 }
@@ -212,17 +219,21 @@ __device__ __forceinline__ void face_fast(const Par &P, const double L[2 + NT],
   }
 }
 
-// Limiter value for the ratio num/den of eq. limiter, 0 for a zero wave.
-template <int LIM> __device__ __forceinline__ double phi_general(double num, double den) {
+// Limiter value for the ratio num/den of eq. limiter, 0 for a zero wave (which
+// divides 1 by 1: 0/0 would take the division's slow path, for a lane without a
+// left neighbour in every warp of the lanes_ forms).
+template <int LIM>
+__device__ __forceinline__ double phi_general(const Unit &U, double num, double den) {
   if (LIM == F64_NONE) return 0.0;
   if (LIM == F64_LW) return den > 0.0 ? 1.0 : 0.0;
-  const double theta = num / den;
-  const double a = 0.5 * (1.0 + theta);
+  const bool on = den > 0.0;
+  const double theta = (on ? num : 1.0) / (on ? den : 1.0);
+  const double a = U.mul(0.5, U.add(theta, 1.0));
   double m = a < 2.0 ? a : 2.0;
-  const double b = 2.0 * theta;
+  const double b = U.add(theta, theta);
   m = m < b ? m : b;
   m = m > 0.0 ? m : 0.0;
-  return den > 0.0 ? m : 0.0;
+  return on ? m : 0.0;
 }
 // den >= 0.  theta >= 3 gives 2, theta <= 0 gives 0; between, the smaller of
 // (1 + theta)/2 and 2 theta, compared as bit patterns.
@@ -252,42 +263,65 @@ __device__ __forceinline__ double phi_fast(const Unit &U, double num, double den
   return int64f::of_bits(m);
 }
 
-// Fluctuations and correction flux of face I between the faces Lf and Rf.
+// Fluctuations and correction flux of face I between the faces Lf and Rf.  In
+// 2D a subsonic face's sums over the families are one term each (the others are
+// exact zeros), which saves twelve of some 210 instructions a cell; in 3D the
+// branch costs the other forms 2 % (145 x 130 x 113 cells, 4 steps: 7.89 ms
+// without, 8.04 with).
 template <int LIM, int NT>
-__device__ __forceinline__ void flux_general(const Face<NT> &I, const Face<NT> &Lf,
-                                             const Face<NT> &Rf, double lam, Flux<NT> &o) {
+__device__ __forceinline__ void flux_general(const Par &P, const Face<NT> &I, const Face<NT> &Lf,
+                                             const Face<NT> &Rf, Flux<NT> &o) {
+  const Unit &U = P.U;
   const double s0 = I.s0, s1 = I.s1, u = I.u;
-  const double sm0 = s0 < 0.0 ? s0 : 0.0, sp0 = s0 > 0.0 ? s0 : 0.0;
-  const double sm1 = s1 < 0.0 ? s1 : 0.0, sp1 = s1 > 0.0 ? s1 : 0.0;
   const double smu = u < 0.0 ? u : 0.0, spu = u > 0.0 ? u : 0.0;
   const bool l0 = s0 > 0.0, l1 = s1 > 0.0, lu = u > 0.0;
-  o.am[0] = sm0 * I.a1 + sm1 * I.a2;
-  o.ap[0] = sp0 * I.a1 + sp1 * I.a2;
-  o.am[1] = sm0 * I.w01 + sm1 * I.w11;
-  o.ap[1] = sp0 * I.w01 + sp1 * I.w11;
-  double d0 = I.a1 * I.a1 + I.w01 * I.w01;
-  double n0 = (l0 ? Lf.a1 : Rf.a1) * I.a1 + (l0 ? Lf.w01 : Rf.w01) * I.w01;
-  double d1 = I.a2 * I.a2 + I.w11 * I.w11;
-  double n1 = (l1 ? Lf.a2 : Rf.a2) * I.a2 + (l1 ? Lf.w11 : Rf.w11) * I.w11;
+  if (NT == 1 && l0 && s1 < 0.0) {
+    o.am[0] = U.mul(s1, I.a2);
+    o.ap[0] = U.mul(s0, I.a1);
+    o.am[1] = U.mul(s1, I.w11);
+    o.ap[1] = U.mul(s0, I.w01);
 #pragma unroll
-  for (int k = 0; k < NT; k++) {
-    o.am[2 + k] = sm0 * I.w0[k] + sm1 * I.w1[k] + smu * I.w2[k];
-    o.ap[2 + k] = sp0 * I.w0[k] + sp1 * I.w1[k] + spu * I.w2[k];
-    d0 = d0 + I.w0[k] * I.w0[k];
-    n0 = n0 + (l0 ? Lf.w0[k] : Rf.w0[k]) * I.w0[k];
-    d1 = d1 + I.w1[k] * I.w1[k];
-    n1 = n1 + (l1 ? Lf.w1[k] : Rf.w1[k]) * I.w1[k];
+    for (int k = 0; k < NT; k++) {
+      o.am[2 + k] = U.add(U.mul(s1, I.w1[k]), U.mul(smu, I.w2[k]));
+      o.ap[2 + k] = U.add(U.mul(s0, I.w0[k]), U.mul(spu, I.w2[k]));
+    }
+  } else {
+    const double sm0 = s0 < 0.0 ? s0 : 0.0, sp0 = s0 > 0.0 ? s0 : 0.0;
+    const double sm1 = s1 < 0.0 ? s1 : 0.0, sp1 = s1 > 0.0 ? s1 : 0.0;
+    o.am[0] = U.add(U.mul(sm0, I.a1), U.mul(sm1, I.a2));
+    o.ap[0] = U.add(U.mul(sp0, I.a1), U.mul(sp1, I.a2));
+    o.am[1] = U.add(U.mul(sm0, I.w01), U.mul(sm1, I.w11));
+    o.ap[1] = U.add(U.mul(sp0, I.w01), U.mul(sp1, I.w11));
+#pragma unroll
+    for (int k = 0; k < NT; k++) {
+      o.am[2 + k] = U.add(U.add(U.mul(sm0, I.w0[k]), U.mul(sm1, I.w1[k])), U.mul(smu, I.w2[k]));
+      o.ap[2 + k] = U.add(U.add(U.mul(sp0, I.w0[k]), U.mul(sp1, I.w1[k])), U.mul(spu, I.w2[k]));
+    }
   }
-  const double as0 = fabs(s0), as1 = fabs(s1), asu = fabs(u);
-  const double c0 = as0 * (1.0 - lam * as0) * phi_general<LIM>(n0, d0);
-  const double c1 = as1 * (1.0 - lam * as1) * phi_general<LIM>(n1, d1);
-  o.G[0] = c0 * I.a1 + c1 * I.a2;
-  o.G[1] = c0 * I.w01 + c1 * I.w11;
+  double d0 = U.add(U.mul(I.a1, I.a1), U.mul(I.w01, I.w01));
+  double n0 = U.add(U.mul(l0 ? Lf.a1 : Rf.a1, I.a1), U.mul(l0 ? Lf.w01 : Rf.w01, I.w01));
+  double d1 = U.add(U.mul(I.a2, I.a2), U.mul(I.w11, I.w11));
+  double n1 = U.add(U.mul(l1 ? Lf.a2 : Rf.a2, I.a2), U.mul(l1 ? Lf.w11 : Rf.w11, I.w11));
 #pragma unroll
   for (int k = 0; k < NT; k++) {
-    const double U = lu ? Lf.w2[k] : Rf.w2[k];
-    const double c2 = asu * (1.0 - lam * asu) * phi_general<LIM>(U * I.w2[k], I.w2[k] * I.w2[k]);
-    o.G[2 + k] = c0 * I.w0[k] + c1 * I.w1[k] + c2 * I.w2[k];
+    d0 = U.add(d0, U.mul(I.w0[k], I.w0[k]));
+    n0 = U.add(n0, U.mul(l0 ? Lf.w0[k] : Rf.w0[k], I.w0[k]));
+    d1 = U.add(d1, U.mul(I.w1[k], I.w1[k]));
+    n1 = U.add(n1, U.mul(l1 ? Lf.w1[k] : Rf.w1[k], I.w1[k]));
+  }
+  // |s| (1 - dt/dx |s|) phi
+  auto coef = [&](double s, double num, double den) {
+    const double as = fabs(s);
+    return U.mul(U.mul(as, U.sub(1.0, U.mul(P.lam, as))), phi_general<LIM>(U, num, den));
+  };
+  const double c0 = coef(s0, n0, d0), c1 = coef(s1, n1, d1);
+  o.G[0] = U.add(U.mul(c0, I.a1), U.mul(c1, I.a2));
+  o.G[1] = U.add(U.mul(c0, I.w01), U.mul(c1, I.w11));
+#pragma unroll
+  for (int k = 0; k < NT; k++) {
+    const double w = lu ? Lf.w2[k] : Rf.w2[k];
+    const double c2 = coef(u, U.mul(w, I.w2[k]), U.mul(I.w2[k], I.w2[k]));
+    o.G[2 + k] = U.add(U.add(U.mul(c0, I.w0[k]), U.mul(c1, I.w1[k])), U.mul(c2, I.w2[k]));
   }
 }
 
@@ -336,12 +370,14 @@ __device__ __forceinline__ void flux_fast(const Par &P, const Face<NT> &I, const
 
 // Cell update of eq. fv-hr.
 template <int NT>
-__device__ __forceinline__ void update_general(double lam, const double q[2 + NT], const double am[],
+__device__ __forceinline__ void update_general(const Par &P, const double q[2 + NT], const double am[],
                                                const double Gr[], const double ap[],
                                                const double Gl[], double o[2 + NT]) {
+  const Unit &U = P.U;
 #pragma unroll
   for (int k = 0; k < 2 + NT; k++)
-    o[k] = q[k] - lam * (am[k] + ap[k]) - lam * (0.5 * Gr[k] - 0.5 * Gl[k]);
+    o[k] = U.sub(U.sub(q[k], U.mul(P.lam, U.add(am[k], ap[k]))),
+                 U.mul(P.lam, U.sub(U.mul(0.5, Gr[k]), U.mul(0.5, Gl[k]))));
 }
 template <int NT>
 __device__ __forceinline__ void update_fast(const Par &P, const double q[2 + NT], const double am[],
@@ -385,7 +421,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
 #pragma unroll
   for (int i = 0; i < CPL; i++) {
     if (FORM) z_fast<NT>(P, q[i], z[i]);
-    else z_general<NT>(q[i], z[i]);
+    else z_general<NT>(P.U, q[i], z[i]);
   }
 #pragma unroll
   for (int k = 0; k < 2 + NT; k++) ql[k] = up1(q[CPL - 1][k]);
@@ -397,7 +433,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
     const double *L = i ? q[i ? i - 1 : 0] : ql, *zL = i ? z[i ? i - 1 : 0] : zl;
     bool nr = false;
     if (FORM) face_fast<FORM, NT>(P, L, zL, q[i], z[i], F[i]);
-    else nr = face_general<NT>(P.beta2, L, zL, q[i], z[i], F[i]);
+    else nr = face_general<NT>(P, L, zL, q[i], z[i], F[i]);
     const int gl = g + i - 1;                      // left cell of the face
     if (i > 0 || lane > 0) {
       if (!FORM && gl >= -2 && gl <= n) nonreal |= nr;
@@ -427,7 +463,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
   for (int i = 0; i < CPL; i++) {
     const Face<NT> &Lf = i ? F[i ? i - 1 : 0] : A, &Rf = i + 1 < CPL ? F[i + 1 < CPL ? i + 1 : 0] : B;
     if (FORM) flux_fast<FORM, LIM, NT>(P, F[i], Lf, Rf, X[i], tiny);
-    else flux_general<LIM, NT>(F[i], Lf, Rf, P.lam, X[i]);
+    else flux_general<LIM, NT>(P, F[i], Lf, Rf, X[i]);
     if (g + i >= flo && g + i <= fhi) {
 #pragma unroll
       for (int k = 0; k < 2 + NT; k++) X[i].G[k] = 0.0;
@@ -445,7 +481,7 @@ __device__ __forceinline__ void lanes_update(const Par &P, const double q[CPL][2
     const double *mr = i + 1 < CPL ? X[i + 1 < CPL ? i + 1 : 0].am : am;
     const double *Gr = i + 1 < CPL ? X[i + 1 < CPL ? i + 1 : 0].G : G;
     if (half) update_fast<NT>(P, q[i], mr, Gr, X[i].ap, X[i].G, o[i]);
-    else update_general<NT>(P.lam, q[i], mr, Gr, X[i].ap, X[i].G, o[i]);
+    else update_general<NT>(P, q[i], mr, Gr, X[i].ap, X[i].G, o[i]);
   }
 }
 
@@ -503,12 +539,12 @@ template <int LIM, int NT> struct March {
                                        bool plain) {
     double z[1 + NT];
     if (FORM) z_fast<NT>(P, q, z);
-    else z_general<NT>(q, z);
+    else z_general<NT>(P.U, q, z);
     if (j > 0) {
       Face<NT> f;
       if (FORM) face_fast<FORM, NT>(P, c1, z1, q, z, f);
       else {
-        const bool nr = face_general<NT>(P.beta2, c1, z1, q, z, f);
+        const bool nr = face_general<NT>(P, c1, z1, q, z, f);
         if (count_real) nonreal |= nr;
       }
       if (j >= 3) {
@@ -519,7 +555,7 @@ template <int LIM, int NT> struct March {
           flux_fast<FORM, LIM, NT>(P, f1, f2, f, X, tiny);
           half = half && !__any_sync(0xffffffffu, tiny);
         } else {
-          flux_general<LIM, NT>(f1, f2, f, P.lam, X);
+          flux_general<LIM, NT>(P, f1, f2, f, X);
         }
         if (plain) {
 #pragma unroll
@@ -528,7 +564,7 @@ template <int LIM, int NT> struct March {
         if (count_speed) speed_max(smax, f1);
         if (j >= 4) {
           if (half && lhalf) update_fast<NT>(P, c2, X.am, X.G, ap, G, out);
-          else update_general<NT>(P.lam, c2, X.am, X.G, ap, G, out);
+          else update_general<NT>(P, c2, X.am, X.G, ap, G, out);
         }
 #pragma unroll
         for (int k = 0; k < 2 + NT; k++) {

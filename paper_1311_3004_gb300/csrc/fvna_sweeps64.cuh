@@ -14,7 +14,7 @@
 //                from the adjacent lanes by warp shuffles.  Twelve warps an SM
 //                are faster than sixteen or eight (2048 x 2048 cells: 1.04,
 //                1.10, 1.37 ms), although the three forms of a step do not
-//                fit their 168 registers (MC limiter: 452 bytes of spill
+//                fit their 168 registers (MC limiter: 444 bytes of spill
 //                stores, 1,368 of spill loads; 9.7 M of 416 M instructions).
 //   k_sweep_yl64 the same for domains of fewer cells: the lanes along x2, a
 //                column of 32 rows at a time, and the block's warps on
