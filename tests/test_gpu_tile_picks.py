@@ -56,6 +56,16 @@ def test_narrow_domains_fp32(nx, ny):
     assert picked <= MARGIN * given, (picked, given)
 
 
+def test_redone_tiles_fp32():
+    """A flow along x2 beyond the subsonic form: every tile of the x2 sweep is
+    marched again by its second kernel, also where the tiles are the shortest."""
+    nx, ny = 700, 370
+    q = _state(nx, ny)
+    q[2] += 0.75 * q[0]
+    picked, given = (_time(_config(fvna.FP32_PERT, 60, ty), nx, ny, q) for ty in (0, 10))
+    assert picked <= MARGIN * given, (picked, given)
+
+
 @pytest.mark.parametrize("precision,nx,ny", [(fvna.FP64, 512, 8), (fvna.FP64, 300, 300),
                                              (fvna.FP32_PERT, 61, 61)])
 def test_tuned_no_slower_than_picked(precision, nx, ny):
