@@ -546,9 +546,10 @@ static int init_impl(const fvna_config *cfg, int n, const fvna_domain *doms,
     CK(cudaMalloc(&c->d_redo, (2 + (size_t)c->nty) * sizeof(int)));
     CK(cudaMemsetAsync(c->d_redo, 0, 2 * sizeof(int), c->stream));
     // 2-row tiles are five times as many: with a block an SM a field whose tiles
-    // are all redone took 103 us a step at 700 x 370 cells, now 51 (10-row tiles
-    // 69), and one without any 27.5 as before
-    c->redo_blocks = c->tile_y < 8 ? 4 * sms : sms;
+    // are all redone took 103 us a step at 700 x 370 cells, now 70 (10-row tiles
+    // 69), and one without any 27.5 as before (four blocks: 51, but 0.3 % on every
+    // step without redone tiles)
+    c->redo_blocks = c->tile_y < 8 ? 2 * sms : sms;
     // x1 sweep, x2 sweep and its second kernel, which ends the step
   }
 
